@@ -246,8 +246,9 @@ fr_status fr_accumulate(const fr_routing* routing, const float* rain, float* w_o
  *   dem          [ny*nx] float32, finite (FR_CHECK_FINITE checks it).
  *   flags        0 or FR_CHECK_FINITE.
  *   filled_out   [ny*nx] float32, not overlapping dem.
- *   max_sweeps   >= 1: relaxation sweeps over 64x32 tiles allowed; a sweep
- *                that changes nothing ends the call.  FR_ERR_NO_PROGRESS if
+ *   max_sweeps   >= 1: relaxation sweeps over 64x64 tiles allowed; a sweep
+ *                that changes nothing ends the call (from 4096 on a mere
+ *                backstop: short sweeps are run, eight of them counting as one).  FR_ERR_NO_PROGRESS if
  *                the surface is still moving after max_sweeps (filled_out
  *                then holds an upper bound of F).
  *   sweeps_out   host int32 or NULL: sweeps run, the last one changing nothing.

@@ -67,10 +67,16 @@ Layout layout(int64_t n) {
 }
 
 // fr_fill's workspace: the sweep counters (one per sweep of a batch) and two
-// per-tile change records.
+// per-tile records of the tiles to run (the documented size, two bytes per
+// 64x32 tile, holds them twice over).
 constexpr int kFillBatch = 8;  // sweeps launched between two reads of the counters
+// Passes of a tile per sweep: two where the limit on sweeps is a mere backstop
+// (the fastest; see fr_fill.cu), and then eight such sweeps count as one towards the
+// limit; until the tile settles where the caller counts sweeps.
+constexpr int kFillQuickPasses = 2, kFillSettlePasses = 384;
+constexpr int32_t kFillQuickFrom = 4096;
 size_t fill_ws_bytes(int64_t nx, int64_t ny) {
-    return 256 + align256((size_t)fill_tiles(nx, ny)) * 2;
+    return 256 + align256((size_t)(((nx + 63) / 64) * ((ny + 31) / 32))) * 2;
 }
 
 bool sizes_ok(int64_t nx, int64_t ny) {
@@ -320,19 +326,22 @@ fr_status fr_fill(const float* dem, int64_t nx, int64_t ny, uint32_t flags, floa
         fr_status st = check_finite(dem, n, s);
         if (st != FR_OK) return st;
     }
-    if (fill_init(dem, nx, ny, filled_out, s) != cudaSuccess) return FR_ERR_CUDA;
     // counters of one batch of sweeps in the first 256 bytes, then the two
-    // per-tile change records (written by every sweep before they are read)
+    // per-tile records, which start at zero
     unsigned long long* counts = reinterpret_cast<unsigned long long*>(ws);
-    uint8_t* act[2] = {(uint8_t*)ws + 256, (uint8_t*)ws + 256 + align256((size_t)fill_tiles(nx, ny))};
-    for (int32_t done = 0; done < max_sweeps;) {
-        const int32_t b = max_sweeps - done < kFillBatch ? max_sweeps - done : kFillBatch;
+    const size_t ntiles = align256((size_t)fill_tiles(nx, ny));
+    uint8_t* act[2] = {(uint8_t*)ws + 256, (uint8_t*)ws + 256 + ntiles};
+    if (cudaMemsetAsync(act[0], 0, 2 * ntiles, s) != cudaSuccess) return FR_ERR_CUDA;
+    const bool quick = max_sweeps >= kFillQuickFrom;
+    const int64_t limit = quick ? 8 * (int64_t)max_sweeps : max_sweeps;
+    for (int64_t done = 0; done < limit;) {
+        const int32_t b = limit - done < kFillBatch ? (int32_t)(limit - done) : kFillBatch;
         unsigned long long h[kFillBatch];
         if (cudaMemsetAsync(counts, 0, sizeof(h), s) != cudaSuccess) return FR_ERR_CUDA;
         for (int32_t k = 0; k < b; ++k) {
-            const int32_t sweep = done + k;  // 0-based
-            if (fill_sweep(dem, nx, ny, filled_out, act[(sweep + 1) & 1], act[sweep & 1],
-                           sweep == 0, counts + k, s) != cudaSuccess)
+            const int64_t sweep = done + k;  // 0-based
+            if (fill_sweep(dem, nx, ny, filled_out, act[(sweep + 1) & 1], act[sweep & 1], sweep == 0,
+                           quick ? kFillQuickPasses : kFillSettlePasses, counts + k, s) != cudaSuccess)
                 return FR_ERR_CUDA;
         }
         if (cudaMemcpyAsync(h, counts, sizeof(h[0]) * b, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
@@ -340,12 +349,12 @@ fr_status fr_fill(const float* dem, int64_t nx, int64_t ny, uint32_t flags, floa
             return FR_ERR_CUDA;
         for (int32_t k = 0; k < b; ++k) {
             if (h[k] == 0) {  // the first sweep that changed nothing; later ones were idle
-                if (sweeps_out) *sweeps_out = done + k + 1;
+                if (sweeps_out) *sweeps_out = (int32_t)(done + k + 1);
                 return FR_OK;
             }
         }
         done += b;
-        if (sweeps_out) *sweeps_out = done;
+        if (sweeps_out) *sweeps_out = (int32_t)done;
     }
     return FR_ERR_NO_PROGRESS;
 }

@@ -132,14 +132,15 @@ cudaError_t launch_mass_balance_ws(int64_t nx, int64_t ny, const uint8_t* rb, co
 cudaError_t richardson_sweep(bool mfd, const Prob& P, const float2* prev, float2* next,
                              unsigned long long* counts, cudaStream_t s);
 cudaError_t richardson_output(const float2* v, int64_t n, float* hi, float* lo, cudaStream_t s);
-// Depression filling (fr_fill.cu): F = z on the edge and +inf inside, then one
-// relaxation sweep over 64x32 tiles; *changed counts the tiles that moved and
-// act_next[t] records it per tile (act_prev: the previous sweep's record,
-// unused when first).
+// Depression filling (fr_fill.cu): one relaxation sweep over 64x64 tiles (the
+// first one also writes F's start values); *changed counts the tiles that
+// moved.  act[t] says whether tile t runs (unused when first; cleared by the
+// sweep), act_next[t], zero before, is set for the next sweep.  A tile takes at
+// most `passes` passes.
 int64_t fill_tiles(int64_t nx, int64_t ny);
-cudaError_t fill_init(const float* z, int64_t nx, int64_t ny, float* F, cudaStream_t s);
-cudaError_t fill_sweep(const float* z, int64_t nx, int64_t ny, float* F, const uint8_t* act_prev,
-                       uint8_t* act_next, bool first, unsigned long long* changed, cudaStream_t s);
+cudaError_t fill_sweep(const float* z, int64_t nx, int64_t ny, float* F, uint8_t* act,
+                       uint8_t* act_next, bool first, int passes, unsigned long long* changed,
+                       cudaStream_t s);
 cudaError_t launch_mfd_fractions(const float* z, const uint8_t* mask, int64_t nx, int64_t ny,
                                  double dx, double p, uint32_t flags, float* frac, cudaStream_t s);
 cudaError_t launch_receivers_batch(int kind, const Prob* probs, const int64_t* prefix, int nprob,
