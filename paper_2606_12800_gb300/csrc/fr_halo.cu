@@ -6,13 +6,11 @@
 // Sec. 2.4, on overlapping subdomains), and only cells whose dependencies
 // reach outside the extended region go to the global phase.  With several
 // receivers per cell (App. A) dependency sets spread wider than D8 basins, so
-// the halo is deeper: at 64x32 + 8 about 0.9 % of the cells of a rough
-// fractal DEM stay global, against about 21 % for the same tiles without a
-// halo.  The tiles are 64x64 (two blocks of about 103 KB and 384 threads per
-// SM, 1.56 region cells per inner cell): smaller tiles that fit more blocks
-// per SM (64x32, 48x48, 56x48, 40x40) were measured slower, their extra halo
-// cells costing more than the occupancy gains; halos of 6 and 10 cells were
-// slower than 8.
+// the halo is deeper: 8 cells leave 0.7 % of the cells of a rough fractal DEM
+// global (6 cells 1.3 %, 4 cells 3.3 %, none about 20 %).  A region of 96x80
+// cells (80x64 inner, 1.5 region cells per inner cell) fills an SM's shared
+// memory with all that its solve reads: values, the fraction of every edge,
+// dependency bytes and the cell list, about 29 bytes a cell.
 //
 // The three modes differ only in the direction of the dependencies:
 //   forward MFD   w_c = r_c    + sum over donors j    of f_{j->c} w_j
@@ -28,43 +26,52 @@
 // the global phase does, so a cell's value does not depend on which kernel
 // computed it.
 //
-// Cells are finalised in a topological order (Sec. 3.2) discovered on the fly,
-// without block barriers: every cell counts its pending in-region
-// dependencies, and the lane whose decrement completes a count owns that
-// cell.  A lane keeps one of the cells it completes and continues with it;
-// the others go to a shared-memory queue from which idle lanes take work.
-// A warp takes only queue slots that a producer has already reserved, so a
-// wait for a slot is the few instructions between the producer's reservation
-// and its store; a warp that finds the queue empty sleeps until new work is
-// queued or no cell is held or queued anywhere in the CTA (the live count).
-// One lane finalises one cell: its (up to eight) dependency terms are loaded
-// side by side and summed in the fixed order, so the result does not depend
-// on which lane computed it or when.
+// Cells are finalised level by level, a topological order (Sec. 3.2): level 0
+// has no dependency, level l + 1 the cells whose last dependency lies in level
+// l.
+//  - The levels are found on bits: one thread holds, for 32 cells of a region
+//    row, the eight masks "has a dependency in direction k" in registers, and a
+//    level is the AND over k of (no dependency, or the neighbour's done bit),
+//    the neighbours' bits being funnel shifts of the nine words around.  That
+//    takes the place of a counter per cell and an atomic per edge.
+//  - Meanwhile the other warps read the fractions, whole rows at a time, into
+//    one slot per edge of the region (an edge carries water one way only).
+//    Reading them from global memory when a cell is solved costs a cache-line
+//    look-up per cell and direction: 3.1 to 4.4 ms of the 8192^2 solve.
+//  - The cells of each level go to a list, packed, so that a level is solved
+//    with full warps.  One lane finalises one cell: its (up to eight)
+//    dependency terms are loaded side by side and summed in the fixed order,
+//    so the result does not depend on which lane computed it.
+// Cells that never become ready depend on cells outside the region (or lie on
+// a cycle of a caller's routing) and are left to the global phase.
+//
+// What bounds it: about 34 levels per region, 500 cycles each to find (two
+// barriers' worth of latency for little work) and 900 to solve (bank conflicts
+// of the scattered reads while levels are wide, latency when they are narrow),
+// 66 K cycles per region in all.  8192^2: 5.37 ms forward and 5.38 adjoint with
+// the queue of ready cells that this replaces (270 K warp instructions per 64x64
+// tile at 14 busy lanes), 2.87 and 3.14 ms now.
 #include "fr_engine.cuh"
 
 namespace fr {
 namespace {
 
 constexpr int kHaloTX = kMfdTileX, kHaloTY = kMfdTileY, kHaloH = 8;
-constexpr int kHaloNT = 384;
+constexpr int kHaloNT = 1024;
 
 struct HaloGeo {
     static constexpr int TX = kHaloTX, TY = kHaloTY, H = kHaloH;
     static constexpr int EX = TX + 2 * H, EY = TY + 2 * H, NE = EX * EY;  // extended region
-    static constexpr int RX = EX + 2, RY = EY + 2, NR = RX * RY;         // plus a one-cell ring
-    static_assert(NE < 65535, "local indices are 16-bit");
-    static_assert(NE % 4 == 0, "state bytes are packed four to a word");
+    static constexpr int RX = EX + 2, RY = EY + 2;                       // plus a one-cell ring
+    static constexpr int CP = EX + 8, NR = CP * RY;  // padded rows: ring cell (rx, ry) at byte ry * CP + rx + 3,
+                                                     // so region cell (ex, ey) at (ey + 1) * CP + ex + 4
+    static constexpr int WR = EX / 32, NWD = WR * EY;        // 32-cell words per row, in all
+    static constexpr int FP = WR + 2, NF = FP * (EY + 2);    // done bits with a border of zero words
+    static constexpr int OW = (NWD + 31) / 32;               // warps that hold words
+    static_assert(EX % 32 == 0 && EX <= 128 && EY <= 128, "rows are whole words; list entries are 7 + 7 bits");
+    static_assert(TX % 4 == 0 && H % 4 == 0, "four-cell groups");
+    static_assert(NWD <= kHaloNT && 32 * NWD <= NR, "a word per thread; the masks fit the receiver bytes' place");
 };
-
-// Directions whose neighbour of region cell (ex, ey) lies inside the region.
-__device__ __forceinline__ uint32_t region_mask(int ex, int ey) {
-    uint32_t in = 0xFFu;
-    if (ex == 0) in &= ~0x64u;                 // W NW SW
-    if (ex == HaloGeo::EX - 1) in &= ~0x91u;   // E NE SE
-    if (ey == 0) in &= ~0x32u;                 // N NE NW
-    if (ey == HaloGeo::EY - 1) in &= ~0xC8u;   // S SW SE
-    return in;
-}
 
 template <Mode M>
 struct HaloMode {
@@ -72,24 +79,62 @@ struct HaloMode {
     static constexpr bool kMfd = (M == Mode::FwdMfd || M == Mode::AdjMfd);
 };
 
+constexpr int kHaloLevels = 64;  // levels found before they are solved (then the next ones)
+
+template <bool MFD>
 struct SmemHalo {
-    static constexpr int NE = HaloGeo::NE, NR = HaloGeo::NR;
-    float vhi[NE];        // value (water or adjoint), leading word
-    float vlo[NE];        // value, trailing word
-    uint32_t st[NE / 4];  // per cell byte: pending non-bare dependencies
-    uint16_t queue[NE];   // ready cells (kSlotEmpty until written); each cell at most once
-    uint8_t rb[NR];       // receiver masks of region + ring (0 outside the grid)
-    uint8_t dm[NE];       // in-region dependencies (donors forward, receivers adjoint)
-    uint8_t tm[NE];       // in-region targets (receivers forward, donors adjoint)
-    uint8_t fin[NE];      // 1 final, 0 pending, 0x0F outside the grid
-    uint8_t gf[NE];       // 1: a dependency chain leaves the region (solved globally)
-    int head;             // queue slots taken
-    int resv;             // queue slots reserved by producers
-    int live;             // cells queued or held by a lane
-    int gave_up;          // a bounded wait ran out
-    unsigned long long done;
+    static constexpr int NE = HaloGeo::NE, NWD = HaloGeo::NWD;
+    union {
+        float2 v[NE];                       // value (water or adjoint), leading and trailing word
+        uint32_t found[kHaloLevels][NWD];   // before the values: the cells of each level
+    };
+    // fraction of each edge of the region (of its higher cell, towards the
+    // lower): E, S, SE and SW of a cell; the other four are its neighbours'
+    float edge[MFD ? 4 : 1][MFD ? NE : 1];
+    uint16_t list[NE];                  // the cells (ey << 7 | ex), level after level
+    uint32_t done[2][HaloGeo::NF];      // done bits by level parity, zero border
+    alignas(8) uint8_t rb[HaloGeo::NR]; // receiver masks of region + ring (0 outside the grid); then the
+                                        // words' dependency masks, direction k at [k * NWD]
+    alignas(4) uint8_t dm[NE];          // dependencies (donors forward, receivers adjoint)
+    int lev[kHaloLevels + 1];           // where level l starts in the list
+    int nlev, cnt;                      // levels found; cells of one more level
+    int wide, narrow;                   // from level `wide` on at most kHaloMid cells each, from `narrow` 32
+    unsigned int ndone;
 };
-constexpr uint16_t kSlotEmpty = 0xFFFFu;
+constexpr int kHaloMid = 256;
+
+// Plane and offset in `edge` of the edge from a cell in direction k.
+__device__ __forceinline__ constexpr int edge_plane(int k) {
+    return k == 0 || k == 2 ? 0 : k == 1 || k == 3 ? 1 : k == 5 || k == 7 ? 2 : 3;  // E/W, N/S, NW/SE, NE/SW
+}
+__device__ __forceinline__ constexpr int edge_off(int k) {
+    return k == 0 || k == 3 || k == 6 || k == 7 ? 0 : offy(k) * HaloGeo::EX + offx(k);
+}
+
+// The byte vectors (left, centre, right neighbours) of the four cells of word
+// w of a padded row.
+struct HRow3 {
+    uint32_t l, c, r;
+};
+__device__ __forceinline__ HRow3 hrow3(const uint32_t* w) {
+    const uint32_t a = w[-1], b = w[0], d = w[1];
+    return {__byte_perm(a, b, 0x6543), b, __byte_perm(b, d, 0x4321)};
+}
+
+// Barrier `id` among the first n threads' warps (n a multiple of 32); the
+// second form returns whether p holds in any thread.
+__device__ __forceinline__ void bar_n(int id, int n) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+__device__ __forceinline__ bool bar_or(int id, int n, bool p) {
+    int r;
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.s32 p, %3, 0;\n bar.red.or.pred q, %1, %2, p;\n selp.s32 %0, 1, 0, q;\n}"
+        : "=r"(r)
+        : "r"(id), "r"(n), "r"((int)p)
+        : "memory");
+    return r != 0;
+}
 
 // Marks the global inner cells of a warp (all 32 lanes call; glob: this
 // lane's cell gi is global): their bits, and list entries reserved with one
@@ -110,60 +155,6 @@ __device__ __forceinline__ void mark_global_cells(const Prob& P, EngineGlobals* 
     }
 }
 
-__device__ __forceinline__ unsigned lanemask_lt() {
-    unsigned m;
-    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
-    return m;
-}
-
-__device__ __forceinline__ int ld_volatile(const int* p) { return *reinterpret_cast<const volatile int*>(p); }
-
-// Warp-aggregated queue append: lane l appends the region cells c + off(k)
-// for the set bits k < 8 of its mask `bits`, and c itself for bit 8.  Lane 0
-// first adds (appended cells - finished) to the live count, then reserves the
-// slots: the count never drops below the cells queued or held, so it reads
-// zero only when the region has no work left.  The cells are stored after a
-// block fence, so a consumer that reads a slot sees what the producer wrote
-// before it.
-__device__ __forceinline__ void queue_push(SmemHalo& S, int c, uint32_t bits, int finished) {
-    const unsigned lane = threadIdx.x & 31u;
-    if (!__any_sync(0xffffffffu, bits != 0)) {
-        // the common step: nothing to queue, only finished cells to count
-        if (lane == 0 && finished) atomicAdd(&S.live, -finished);
-        return;
-    }
-    const unsigned lt = lanemask_lt();
-    const uint32_t n = (uint32_t)__popc(bits);
-    // exclusive prefix of n (at most 9) over the lanes, from the ballots of its bits
-    uint32_t pre = 0, tot = 0;
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-        const unsigned v = __ballot_sync(0xffffffffu, (n >> b) & 1u);
-        pre += (uint32_t)__popc(v & lt) << b;
-        tot += (uint32_t)__popc(v) << b;
-    }
-    int base = 0;
-    if (lane == 0) {
-        if ((int)tot != finished) atomicAdd(&S.live, (int)tot - finished);
-        if (tot) base = atomicAdd(&S.resv, (int)tot);
-    }
-    if (tot == 0) return;
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if (bits) {
-        __threadfence_block();
-        int slot = base + (int)pre;
-        for (uint32_t m = bits; m; m &= m - 1) {
-            const int k = __ffs(m) - 1;
-            const int cell = k == 8 ? c : c + offy(k) * HaloGeo::EX + offx(k);
-            if (slot < HaloGeo::NE)
-                reinterpret_cast<volatile uint16_t*>(S.queue)[slot] = (uint16_t)cell;
-            else
-                S.gave_up = 1;  // unreachable: each cell is queued at most once
-            ++slot;
-        }
-    }
-}
-
 // Problem and tile of this CTA in a batched launch: the problem whose tiles
 // [prefix[p], prefix[p+1]) hold blockIdx.x.
 __device__ __forceinline__ int batch_problem_halo(const int64_t* __restrict__ prefix, int nprob,
@@ -180,19 +171,20 @@ __device__ __forceinline__ int batch_problem_halo(const int64_t* __restrict__ pr
 }
 
 template <Mode M, bool BATCH>
-__global__ void __launch_bounds__(kHaloNT, 2) k_local_halo(Prob Pone, EngineGlobals* G,
+__global__ void __launch_bounds__(kHaloNT, 1) k_local_halo(Prob Pone, EngineGlobals* G,
                                                            const Prob* __restrict__ probs,
                                                            const int64_t* __restrict__ prefix,
-                                                           int nprob, unsigned long long limit_ns) {
+                                                           int nprob) {
     using HM = HaloMode<M>;
     constexpr int TX = HaloGeo::TX, TY = HaloGeo::TY, H = HaloGeo::H;
-    constexpr int EX = HaloGeo::EX, NE = HaloGeo::NE;
-    constexpr int RX = HaloGeo::RX;
-    constexpr int NT = kHaloNT;
+    constexpr int EX = HaloGeo::EX, EY = HaloGeo::EY;
+    constexpr int RX = HaloGeo::RX, RY = HaloGeo::RY;
+    constexpr int WR = HaloGeo::WR, NWD = HaloGeo::NWD, FP = HaloGeo::FP;
+    constexpr int NT = kHaloNT, NW = NT / 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    SmemHalo& S = *reinterpret_cast<SmemHalo*>(smem_raw);
-    uint8_t* stb = reinterpret_cast<uint8_t*>(S.st);
-    const int tid = threadIdx.x;
+    using Sm = SmemHalo<HM::kMfd>;
+    Sm& S = *reinterpret_cast<Sm*>(smem_raw);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     int64_t lt = (int64_t)blockIdx.x;
     const int pid = BATCH ? batch_problem_halo(prefix, nprob, lt) : 0;
     const Prob& P = BATCH ? probs[pid] : Pone;
@@ -200,323 +192,417 @@ __global__ void __launch_bounds__(kHaloNT, 2) k_local_halo(Prob Pone, EngineGlob
     const int64_t ty = lt / tiles_x, tx = lt - ty * tiles_x;
     const int64_t x0 = tx * TX, y0 = ty * TY;
     const int64_t ox = x0 - H - 1, oy = y0 - H - 1;  // ring origin (may be negative)
-    if (tid == 0) {
-        S.head = S.resv = S.live = S.gave_up = 0;
-    }
-
-    // The phases below walk the region row by row: warp w takes rows w,
-    // w + NW, ...; lane l takes columns l, l + 32, ...  A tile whose ring lies
-    // inside the grid skips the bounds checks.
-    constexpr int NW = NT / 32;
-    constexpr int EY = HaloGeo::EY, RY = HaloGeo::RY;
-    const int warp = tid >> 5, lane_id = tid & 31;
+    // a tile whose ring lies inside the grid skips the bounds checks
     const bool interior = ox >= 0 && oy >= 0 && ox + RX <= P.nx && oy + RY <= P.ny;
 
     // ---- region + ring: receiver masks
-    if (interior) {
-        for (int ry = warp; ry < RY; ry += NW) {
-            const uint8_t* src = P.rb + (oy + ry) * P.nx + ox;
-            for (int rx = lane_id; rx < RX; rx += 32)
-                S.rb[ry * RX + rx] = (uint8_t)recv_mask<HM::kMfd>(__ldg(src + rx));
+    const bool vec = HM::kMfd && interior && x0 >= H + 4 && x0 + EX - H + 4 <= P.nx && (P.nx & 3) == 0 &&
+                     ((uintptr_t)P.rb & 3) == 0;
+    if (vec) {
+        // whole padded rows (byte b is grid x = x0 - H - 4 + b), a word a lane
+        constexpr int U = (RY + NW - 1) / NW, W4 = HaloGeo::CP / 4;
+        static_assert(W4 <= 32, "a row of words per warp");
+        uint32_t m[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int ry = warp + u * NW;
+            m[u] = 0;
+            if (ry < RY && lane < W4)
+                m[u] = __ldg(reinterpret_cast<const uint32_t*>(P.rb + (oy + ry) * P.nx + (x0 - H - 4)) + lane);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int ry = warp + u * NW;
+            if (ry < RY && lane < W4) reinterpret_cast<uint32_t*>(S.rb)[ry * W4 + lane] = m[u];
         }
     } else {
-        for (int ry = warp; ry < RY; ry += NW) {
-            const int64_t gy = oy + ry;
-            for (int rx = lane_id; rx < RX; rx += 32) {
-                const int64_t gx = ox + rx;
-                uint8_t m = 0;
-                if (gx >= 0 && gy >= 0 && gx < P.nx && gy < P.ny)
-                    m = (uint8_t)(recv_mask<HM::kMfd>(rd_rb(P, gy * P.nx + gx)) & grid_mask(gx, gy, P.nx, P.ny));
-                S.rb[ry * RX + rx] = m;
+        constexpr int U = 3, C = (RX + 31) / 32;
+        for (int r0 = warp; r0 < RY; r0 += U * NW) {
+            uint8_t m[U][C];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int ry = r0 + u * NW;
+                const int64_t gy = oy + ry;
+#pragma unroll
+                for (int q = 0; q < C; ++q) {
+                    const int rx = lane + 32 * q;
+                    const int64_t gx = ox + rx;
+                    m[u][q] = HM::kMfd ? 0 : kSink;
+                    if (ry < RY && rx < RX && (interior || (gx >= 0 && gy >= 0 && gx < P.nx && gy < P.ny)))
+                        m[u][q] = rd_rb(P, gy * P.nx + gx);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int ry = r0 + u * NW;
+#pragma unroll
+                for (int q = 0; q < C; ++q) {
+                    const int rx = lane + 32 * q;
+                    if (ry >= RY || rx >= RX) continue;
+                    uint32_t b = recv_mask<HM::kMfd>(m[u][q]);
+                    if (!interior) b &= grid_mask(ox + rx, oy + ry, P.nx, P.ny);
+                    S.rb[ry * HaloGeo::CP + rx + 3] = (uint8_t)b;
+                }
             }
         }
     }
+    for (int i = tid; i < HaloGeo::NF; i += NT) S.done[0][i] = S.done[1][i] = 0u;
+    if (tid == 0) S.ndone = 0;
+    __syncthreads();
+
+    // ---- dependency bytes, four cells a step
+    for (int g = tid; g < HaloGeo::NE / 4; g += NT) {
+        const int ey = g / (EX / 4), ex = (g - ey * (EX / 4)) * 4;
+        const uint32_t* row = reinterpret_cast<const uint32_t*>(S.rb + (ey + 1) * HaloGeo::CP + ex + 4);
+        uint32_t d;
+        if constexpr (HM::kAdj) {
+            d = row[0];
+        } else {
+            // the donor in direction k has receiver bit opp(k) = k ^ 2 set
+            const HRow3 up = hrow3(row - HaloGeo::CP / 4), mid = hrow3(row), dn = hrow3(row + HaloGeo::CP / 4);
+            d = ((mid.r >> 2) & 0x01010101u) | ((up.c >> 2) & 0x02020202u);
+            d |= ((mid.l << 2) & 0x04040404u) | ((dn.c << 2) & 0x08080808u);
+            d |= ((up.r >> 2) & 0x10101010u) | ((up.l >> 2) & 0x20202020u);
+            d |= ((dn.l << 2) & 0x40404040u) | ((dn.r << 2) & 0x80808080u);
+        }
+        reinterpret_cast<uint32_t*>(S.dm)[g] = d;
+    }
+    __syncthreads();
+
+    // ---- this thread's word: dependency masks by direction (a transposition of
+    // the 32 bytes), the cells that can become ready, level 0
+    uint32_t open = 0, fin = 0, ndep[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    const bool owner = tid < NWD;
+    int fw = 0, wy = 0, wx = 0;  // index of the word's done bits; its first cell
+    uint32_t* const dep_s = reinterpret_cast<uint32_t*>(S.rb) + tid;
+    if (owner) {
+        wy = tid / WR;
+        wx = (tid - wy * WR) * 32;
+        fw = (wy + 1) * FP + (tid - wy * WR) + 1;
+        uint32_t dep[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const uint32_t b = reinterpret_cast<const uint32_t*>(S.dm + wy * EX + wx)[q];
+#pragma unroll
+            for (int k = 0; k < 8; ++k)  // bits k of the four bytes, gathered at bits 28..31
+                dep[k] |= ((((b >> k) & 0x01010101u) * 0x10204080u) >> 28) << (4 * q);
+        }
+        const int64_t gy = oy + wy + 1, gx = ox + wx + 1;
+        uint32_t valid = gy >= 0 && gy < P.ny ? ~0u : 0u;
+        if (gx < 0) valid = gx > -32 ? valid & (~0u << -gx) : 0u;
+        if (gx + 32 > P.nx) valid = gx < P.nx ? valid & (~0u >> (gx + 32 - P.nx)) : 0u;
+        uint32_t shut = 0;  // a dependency outside the region
+        if (wy == 0) shut |= dep[1] | dep[4] | dep[5];
+        if (wy == EY - 1) shut |= dep[3] | dep[6] | dep[7];
+        if (wx == 0) shut |= (dep[2] | dep[5] | dep[6]) & 1u;
+        if (wx == EX - 32) shut |= (dep[0] | dep[4] | dep[7]) & 0x80000000u;
+        open = valid & ~shut;
+        fin = open & ~(dep[0] | dep[1] | dep[2] | dep[3] | dep[4] | dep[5] | dep[6] | dep[7]);
+        S.done[0][fw] = fin;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) ndep[k] = ~dep[k];
+    }
+    // ---- the edges' fractions, by the warps that hold no bits, while the
+    // others find the levels: each cell's row of eight goes to the edges it
+    // gives to (the float4s of a region row are contiguous)
     if constexpr (HM::kMfd) {
-        // warm L2 with the region's fractions, which the dependency pulls read
-        // a few at a time: one prefetch per 128-byte line of every region row
-        const int64_t gx0 = ox + 1 < 0 ? 0 : ox + 1;
-        const int64_t gx1 = ox + 1 + EX > P.nx ? P.nx : ox + 1 + EX;
-        if (gx1 > gx0) {
-            const int lines = (int)(((gx1 - gx0) * 32 + 127) / 128) + 1;
-            for (int ry = warp; ry < EY; ry += NW) {
-                const int64_t gy = oy + 1 + ry;
-                if (gy < 0 || gy >= P.ny) continue;
-                const char* row = reinterpret_cast<const char*>(P.frac + (gy * P.nx + gx0) * 8);
-                const char* end = reinterpret_cast<const char*>(P.frac + (gy * P.nx + gx1) * 8);
-                for (int q = lane_id; q < lines; q += 32) {
-                    const char* a = row + 128 * q;
-                    if (a < end) asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
-                }
-            }
-        }
-    }
-    __syncthreads();
-
-    // ---- per region cell: dependencies and targets, bare / global flags,
-    // initial value (rain forward; gbar adjoint)
-    for (int ey = warp; ey < EY; ey += NW) {
-        const int64_t gy = oy + ey + 1;
-        const bool row_in = gy >= 0 && gy < P.ny;
-        for (int ex = lane_id; ex < EX; ex += 32) {
-            const int c = ey * EX + ex;
-            const int r = (ey + 1) * RX + ex + 1;
-            const int64_t gx = ox + ex + 1;
-            uint8_t dmr = 0, tmr = 0, fin = 0x0F, b = 0;
-            float vh = 0.0f, vl = 0.0f;
-            if (interior || (row_in && gx >= 0 && gx < P.nx)) {
-                const int64_t gi = gy * P.nx + gx;
-                uint32_t don = 0;
+        if (warp >= HaloGeo::OW) {
+            constexpr int N4 = 2 * HaloGeo::NE, STEP = NT - HaloGeo::OW * 32, U = 4;
+            for (int i0 = tid - HaloGeo::OW * 32; i0 < N4; i0 += U * STEP) {
+                float4 f[U];
 #pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    don |= (uint32_t)((S.rb[r + offy(k) * RX + offx(k)] >> opp(k)) & 1u) << k;
-                const uint32_t rcv = S.rb[r];
-                const uint32_t dep = HM::kAdj ? rcv : don;
-                const uint32_t tgt = HM::kAdj ? don : rcv;
-                const uint32_t in = region_mask(ex, ey);
-                dmr = (uint8_t)(dep & in);
-                tmr = (uint8_t)(tgt & in);
-                b = (dep & ~in) ? (uint8_t)1 : (uint8_t)0;
-                fin = dep == 0;
-                if constexpr (!HM::kAdj) {
-                    vh = P.init ? rd_in(P.init, P, gi, 8) : 1.0f;
-                } else if (P.init) {
-                    vh = rd_in(P.init, P, gi, 8);
-                } else if (!rcv) {
-                    // L = sum over sinks of w^2: gbar = 2 w at a sink, 0 elsewhere
-                    vh = __fmul_rn(2.0f, rd_in(P.wf, P, gi, 9));
-                    vl = P.wf_lo ? __fmul_rn(2.0f, rd_in(P.wf_lo, P, gi, 10)) : 0.0f;
+                for (int u = 0; u < U; ++u) {
+                    const int i = i0 + u * STEP, c = i >> 1, ey = c / EX, ex = c - ey * EX;
+                    const int64_t gx = ox + ex + 1, gy = oy + ey + 1;
+                    f[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (i < N4 && (interior || (gx >= 0 && gy >= 0 && gx < P.nx && gy < P.ny)))
+                        f[u] = __ldg(reinterpret_cast<const float4*>(P.frac) + 2 * (gy * P.nx + gx) + (i & 1));
                 }
-            }
-            S.dm[c] = dmr;
-            S.tm[c] = tmr;
-            S.fin[c] = fin;
-            S.gf[c] = b;
-            S.queue[c] = kSlotEmpty;
-            S.vhi[c] = vh;
-            S.vlo[c] = vl;
-        }
-    }
-    __syncthreads();
-
-    // ---- counts of non-bare in-region dependencies; cells with none are
-    // ready at once and start the queue (every lane of a warp runs the same
-    // number of column steps, as queue_push needs)
-    for (int ey = warp; ey < EY; ey += NW) {
-        for (int ex0 = 0; ex0 < EX; ex0 += 32) {
-            const int ex = ex0 + lane_id;
-            const int c = ey * EX + ex;
-            uint32_t start = 0;
-            if (ex < EX) {
-                uint32_t n = 0;
-                if (S.fin[c] == 0) {
-                    const uint32_t dm = S.dm[c];
 #pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        n += ((dm >> k) & 1u) && S.fin[c + offy(k) * EX + offx(k)] != 1;
-                    start = n == 0;
-                }
-                stb[c] = (uint8_t)n;
-            }
-            queue_push(S, c, start ? 0x100u : 0u, 0);  // bit 8: the cell itself
-        }
-    }
-    __syncthreads();
-
-    // ---- dataflow over the region: finalise ready cells, pass readiness on
-    {
-        const unsigned lane = tid & 31u;
-        int cur = -1;                 // the cell this lane holds
-        unsigned long long idle_since = 0;
-        for (;;) {
-            // idle lanes take reserved queue slots, in lane order
-            const unsigned idle = __ballot_sync(0xffffffffu, cur < 0);
-            if (idle) {
-                int h = 0, n = 0;
-                if (lane == 0) {
-                    int hh = ld_volatile(&S.head);
-                    for (int tries = 0; tries < 4096; ++tries) {
-                        const int avail = ld_volatile(&S.resv) - hh;
-                        n = avail < __popc(idle) ? avail : __popc(idle);
-                        if (n <= 0) {
-                            n = 0;
-                            break;
-                        }
-                        const int prev = atomicCAS(&S.head, hh, hh + n);
-                        if (prev == hh) break;
-                        hh = prev;
-                        n = 0;
-                    }
-                    h = hh;
-                }
-                h = __shfl_sync(0xffffffffu, h, 0);
-                n = __shfl_sync(0xffffffffu, n, 0);
-                const int rank = __popc(idle & lanemask_lt());
-                if (cur < 0 && rank < n && h + rank < NE) {
-                    const volatile uint16_t* q = reinterpret_cast<const volatile uint16_t*>(S.queue);
-                    uint16_t v = q[h + rank];
-                    if (v == kSlotEmpty) {
-                        // the producer reserved this slot and stores it next
-                        const unsigned long long t0 = global_ns();
-                        while ((v = q[h + rank]) == kSlotEmpty)
-                            if (global_ns() - t0 > limit_ns) break;
-                    }
-                    if (v != kSlotEmpty) cur = v;
-                    else S.gave_up = 1;
-                }
-            }
-            if (!__any_sync(0xffffffffu, cur >= 0)) {
-                // nothing held here and nothing queued: done when no cell is
-                // held or queued anywhere, else wait for more work (lane 0
-                // decides for the warp)
-                int stop = 0;
-                if (lane == 0) {
-                    if (ld_volatile(&S.live) == 0) {
-                        stop = 1;
+                for (int u = 0; u < U; ++u) {
+                    const int i = i0 + u * STEP, c = i >> 1, ey = c / EX, ex = c - ey * EX;
+                    if (i >= N4) break;
+                    uint32_t m = S.rb[(ey + 1) * HaloGeo::CP + ex + 4];
+                    if (ex == 0) m &= ~0x64u;       // edges that leave the region: W NW SW
+                    if (ex == EX - 1) m &= ~0x91u;  // E NE SE
+                    if (ey == 0) m &= ~0x32u;       // N NE NW
+                    if (ey == EY - 1) m &= ~0xC8u;  // S SW SE
+                    if (i & 1) {
+                        if (m & 0x10u) S.edge[3][c + edge_off(4)] = f[u].x;
+                        if (m & 0x20u) S.edge[2][c + edge_off(5)] = f[u].y;
+                        if (m & 0x40u) S.edge[3][c] = f[u].z;
+                        if (m & 0x80u) S.edge[2][c] = f[u].w;
                     } else {
-                        const unsigned long long t = global_ns();
-                        if (!idle_since) {
-                            idle_since = t;
-                        } else if (t - idle_since > limit_ns) {
-                            S.gave_up = 1;
-                            stop = 1;
-                        }
+                        if (m & 0x01u) S.edge[0][c] = f[u].x;
+                        if (m & 0x02u) S.edge[1][c + edge_off(1)] = f[u].y;
+                        if (m & 0x04u) S.edge[0][c + edge_off(2)] = f[u].z;
+                        if (m & 0x08u) S.edge[1][c] = f[u].w;
                     }
-                }
-                if (__shfl_sync(0xffffffffu, stop, 0)) break;
-                __nanosleep(128);
-                continue;
-            }
-            idle_since = 0;
-            uint32_t ready = 0;  // codes of targets this lane completed
-            if (cur >= 0) {
-                const int c = cur;
-                __threadfence_block();  // acquire: the dependencies' values and flags
-                const bool glob = S.gf[c] != 0;
-                if (!glob) {
-                    // dependency terms, loaded side by side, accumulated in
-                    // the fixed order of df_dot8
-                    const uint32_t dm = S.dm[c];
-                    const float* fb = nullptr;
-                    int64_t row = 0;
-                    if constexpr (HM::kMfd) {
-                        const int ey = c / EX, ex = c - ey * EX;
-                        fb = P.frac + ((oy + ey + 1) * P.nx + (ox + ex + 1)) * 8;
-                        row = P.nx * 8;
-                    }
-                    float f[8];
-                    df vv[8];
-                    float4 f0 = make_float4(0.f, 0.f, 0.f, 0.f), f1 = f0;
-                    if constexpr (HM::kMfd && HM::kAdj) {
-                        // adjoint: c's own fractions towards its receivers, one 32-byte row
-                        f0 = __ldg(reinterpret_cast<const float4*>(fb));
-                        f1 = __ldg(reinterpret_cast<const float4*>(fb) + 1);
-                    }
-                    const float own[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        f[k] = 0.0f;
-                        vv[k] = df_make(0.0f);
-                        if (!((dm >> k) & 1u)) continue;
-                        const int j = c + offy(k) * EX + offx(k);
-                        vv[k] = {S.vhi[j], S.vlo[j]};
-                        if constexpr (HM::kMfd) {
-                            // forward: the donor's fraction towards c
-                            f[k] = HM::kAdj ? own[k] : __ldg(fb + offy(k) * row + (offx(k) * 8 + opp(k)));
-                        } else {
-                            f[k] = 1.0f;
-                        }
-                    }
-                    const df v = df_dot8(df{S.vhi[c], S.vlo[c]}, f, vv);
-                    S.vhi[c] = v.hi;
-                    S.vlo[c] = v.lo;
-                }
-                S.fin[c] = 1;
-                // targets: pass on the global flag, then count down (release)
-                const uint32_t tm = S.tm[c];
-                if (glob) {
-#pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        if ((tm >> k) & 1u) S.gf[c + offy(k) * EX + offx(k)] = 1;
-                }
-                __threadfence_block();
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    if (!((tm >> k) & 1u)) continue;
-                    const int t = c + offy(k) * EX + offx(k);
-                    const uint32_t sh = 8u * (uint32_t)(t & 3);
-                    const uint32_t old = atomicSub(&S.st[t >> 2], 1u << sh);
-                    if (((old >> sh) & 0x0Fu) == 1u) ready |= 1u << k;
                 }
             }
-            // keep one completed target, queue the rest; then the live count
-            // gains the queued cells and loses the finished ones
-            int next = -1;
-            if (ready) {
-                const int k = __ffs(ready) - 1;
-                ready &= ready - 1;
-                next = cur + offy(k) * EX + offx(k);
+        }
+    }
+
+    // ---- up to kHaloLevels levels, by the warps that hold bits
+    int cur = 0;
+    // the cells of this thread's word that level `cur` makes ready
+    auto next_ready = [&](const uint32_t (&nd)[8]) -> uint32_t {
+        uint32_t ready = open & ~fin;
+        if (!ready) return 0u;
+        const uint32_t* d = S.done[cur] + fw;
+        const uint32_t ul = d[-FP - 1], uc = d[-FP], ur = d[-FP + 1];
+        const uint32_t ml = d[-1], mr = d[1];
+        const uint32_t dl = d[FP - 1], dc = d[FP], dr = d[FP + 1];
+        // bit x of each: the neighbour of cell x in that direction is done
+        ready &= (nd[0] | __funnelshift_r(fin, mr, 1)) & (nd[1] | uc);
+        ready &= (nd[2] | __funnelshift_l(ml, fin, 1)) & (nd[3] | dc);
+        ready &= (nd[4] | __funnelshift_r(uc, ur, 1)) & (nd[5] | __funnelshift_l(ul, uc, 1));
+        ready &= (nd[6] | __funnelshift_l(dl, dc, 1)) & (nd[7] | __funnelshift_r(dc, dr, 1));
+        return ready;
+    };
+    if (warp < HaloGeo::OW) {
+        constexpr int NO = HaloGeo::OW * 32;
+        int l = 0;
+        bar_n(1, NO);  // the done bits of level 0
+        for (; l < kHaloLevels; ++l) {
+            const uint32_t ready = next_ready(ndep);
+            fin |= ready;
+            cur ^= 1;
+            if (owner) {
+                S.done[cur][fw] = fin;
+                S.found[l][tid] = ready;
             }
-            const unsigned fin_w = __ballot_sync(0xffffffffu, cur >= 0 && next < 0);
-            queue_push(S, cur, ready, __popc(fin_w));
-            cur = next;
+            if (!bar_or(1, NO, ready != 0)) break;
+        }
+        if (tid == 0) {
+            S.nlev = l;
+            S.cnt = 0;
         }
     }
     __syncthreads();
+    const int nlev = S.nlev;
+    // the masks move to the receiver bytes' place (needed only if there are
+    // more levels)
+    if (owner && nlev == kHaloLevels) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) dep_s[k * NWD] = ndep[k];
+    }
+    // ---- initial values (rain forward; gbar adjoint): loads
+    constexpr int NV = (HaloGeo::NE + NT - 1) / NT;
+    df vi[NV];
+#pragma unroll
+    for (int u = 0; u < NV; ++u) {
+        const int c = tid + u * NT, ey = c / EX, ex = c - ey * EX;
+        const int64_t gx = ox + ex + 1, gy = oy + ey + 1, gi = gy * P.nx + gx;
+        vi[u] = df_make(0.0f);
+        if (c >= HaloGeo::NE || !(interior || (gx >= 0 && gy >= 0 && gx < P.nx && gy < P.ny))) continue;
+        if constexpr (!HM::kAdj) {
+            vi[u].hi = P.init ? rd_in(P.init, P, gi, 8) : 1.0f;
+        } else if (P.init) {
+            vi[u].hi = rd_in(P.init, P, gi, 8);
+        } else if (!S.dm[c]) {
+            // L = sum over sinks of w^2: gbar = 2 w at a sink, 0 elsewhere
+            vi[u].hi = __fmul_rn(2.0f, rd_in(P.wf, P, gi, 9));
+            vi[u].lo = P.wf_lo ? __fmul_rn(2.0f, rd_in(P.wf_lo, P, gi, 10)) : 0.0f;
+        }
+    }
+    // ---- the levels' cells, packed: a warp per level (two at most) counts,
+    // the counts become list positions, the warp writes
+    {
+        constexpr int LW = kHaloLevels / NW, WPL = (NWD + 31) / 32;
+        static_assert(LW * NW == kHaloLevels, "levels per warp");
+        int mine[LW];
+#pragma unroll
+        for (int q = 0; q < LW; ++q) {
+            const int l = warp + q * NW;
+            int n = 0;
+            if (l < nlev) {
+#pragma unroll
+                for (int j = 0; j < WPL; ++j)
+                    if (j * 32 + lane < NWD) n += __popc(S.found[l][j * 32 + lane]);
+            }
+            mine[q] = n;
+            n = __reduce_add_sync(0xffffffffu, n);
+            if (lane == 0) S.lev[l + 1] = n;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            int base = 0, wide = 0, narrow = 0;
+#pragma unroll
+            for (int q = 0; q < kHaloLevels / 32; ++q) {
+                const int n = S.lev[32 * q + lane + 1];
+                int incl = n;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int u = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += u;
+                }
+                S.lev[32 * q + lane + 1] = base + incl;
+                base += __shfl_sync(0xffffffffu, incl, 31);
+                const unsigned bw = __ballot_sync(0xffffffffu, n > kHaloMid), bn = __ballot_sync(0xffffffffu, n > 32);
+                if (bw) wide = 32 * q + 32 - __clz(bw);
+                if (bn) narrow = 32 * q + 32 - __clz(bn);
+            }
+            if (lane == 0) {
+                S.lev[0] = 0;
+                S.wide = wide;
+                S.narrow = narrow;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < LW; ++q) {
+            const int l = warp + q * NW;
+            if (l >= nlev) break;
+            int incl = mine[q];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += u;
+            }
+            int pos = S.lev[l] + incl - mine[q];
+#pragma unroll
+            for (int j = 0; j < WPL; ++j) {
+                const int w = j * 32 + lane, y = w / WR;
+                if (w >= NWD) break;
+                const int e = y << 7 | (w - y * WR) * 32;
+                for (uint32_t m = S.found[l][w]; m; m &= m - 1) S.list[pos++] = (uint16_t)(e + __ffs(m) - 1);
+            }
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < NV; ++u) {
+        const int c = tid + u * NT;
+        if (c >= HaloGeo::NE) break;
+        // a cell without dependencies is final: as a sum without terms leaves it
+        if (HM::kAdj && !S.dm[c]) vi[u] = df_norm(vi[u].hi, vi[u].lo);
+        S.v[c] = make_float2(vi[u].hi, vi[u].lo);
+    }
+    __syncthreads();
+    // ---- the levels in order: all warps, then eight, then one as the levels
+    // shrink
+    auto solve = [&](int c, uint32_t m) {
+        float f[8];
+        df vv[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            f[k] = 0.0f;
+            vv[k] = df_make(0.0f);
+            if (!((m >> k) & 1u)) continue;
+            const float2 a = S.v[c + offy(k) * EX + offx(k)];
+            vv[k] = {a.x, a.y};
+            if constexpr (HM::kMfd) f[k] = S.edge[edge_plane(k)][c + edge_off(k)];
+            else f[k] = 1.0f;
+        }
+        const float2 o = S.v[c];
+        const df v = df_dot8(df{o.x, o.y}, f, vv);
+        S.v[c] = make_float2(v.hi, v.lo);
+    };
+    auto cell_of = [&](int i) {
+        const int x = S.list[i];
+        return (x >> 7) * EX + (x & 127);
+    };
+    {
+        int l = 0;
+        for (int stage = 0; stage < 3; ++stage) {
+            const int nthr = stage == 0 ? NT : stage == 1 ? kHaloMid : 32;
+            const int end = stage == 0 ? S.wide : stage == 1 ? S.narrow : nlev;
+            if (tid >= nthr) break;
+            int e = -1;
+            uint32_t dm = 0;
+            auto load = [&](int lv) {  // this thread's cell of level lv
+                e = -1;
+                if (lv >= end) return;
+                const int i = S.lev[lv] + tid;
+                if (i >= S.lev[lv + 1]) return;
+                e = cell_of(i);
+                dm = S.dm[e];
+            };
+            load(l);
+            for (; l < end; ++l) {
+                if (e >= 0) {
+                    solve(e, dm);
+                    for (int i = S.lev[l] + tid + nthr; i < S.lev[l + 1]; i += nthr) {
+                        const int c = cell_of(i);
+                        solve(c, S.dm[c]);
+                    }
+                }
+                load(l + 1);
+                if (nthr == NT) __syncthreads();
+                else if (nthr == kHaloMid) bar_n(2, kHaloMid);
+                else __syncwarp();
+            }
+        }
+    }
+    __syncthreads();
+    // ---- chains longer than kHaloLevels (not on rough terrain): level by level
+    while (nlev == kHaloLevels) {
+        if (warp < HaloGeo::OW) {
+            uint32_t nd[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) nd[k] = owner ? dep_s[k * NWD] : 0u;
+            const uint32_t ready = next_ready(nd);
+            fin |= ready;
+            cur ^= 1;
+            if (owner) S.done[cur][fw] = fin;
+            if (ready) {
+                int pos = atomicAdd(&S.cnt, __popc(ready));
+                for (uint32_t m = ready; m; m &= m - 1) S.list[pos++] = (uint16_t)(wy << 7 | (wx + __ffs(m) - 1));
+            }
+        }
+        __syncthreads();
+        const int n = S.cnt;
+        if (n == 0) break;
+        for (int i = tid; i < n; i += NT) {
+            const int c = cell_of(i);
+            solve(c, S.dm[c]);
+        }
+        __syncthreads();
+        if (tid == 0) S.cnt = 0;
+        __syncthreads();
+    }
+    if (owner) S.done[0][fw] = fin;
+    __syncthreads();
 
-    // ---- inner tile: publish final cells, list global ones (every lane of a
-    // warp runs the same steps, as mark_global_cells needs)
-    unsigned long long done = 0;
+    // ---- inner tile: publish final cells, list the others as global (every
+    // lane of a warp runs the same steps, as mark_global_cells needs).  The
+    // trailing word goes out for every cell: 4 bytes more per cell cost less
+    // than finding the cells the global phase will pull from.
+    const uint32_t* fd = S.done[0];
+    unsigned done = 0;
     for (int ly = warp; ly < TY; ly += NW) {
         const int64_t gy = y0 + ly;
         for (int lx0 = 0; lx0 < TX; lx0 += 32) {  // warp-uniform steps
-            const int lx = lx0 + lane_id;
+            const int lx = lx0 + lane;
             const int64_t gx = x0 + lx;
             const bool in_grid = lx < TX && gx < P.nx && gy < P.ny;
-            const int c = (ly + H) * EX + (lx < TX ? lx : 0) + H;
+            const int ex = lx + H, ey = ly + H;
             const int64_t gi = gy * P.nx + gx;
-            const bool glob = in_grid && S.gf[c];
-            mark_global_cells(P, G, gi, pid, glob);
-            // cells never reached (a cycle in a caller's routing) stay unpublished
-            if (!in_grid || glob || S.fin[c] != 1) continue;
+            const bool fin1 = in_grid && ((fd[(ey + 1) * FP + (ex >> 5) + 1] >> (ex & 31)) & 1u);
+            mark_global_cells(P, G, gi, pid, in_grid && !fin1);
+            if (!fin1) continue;
             ++done;
-            wr_f(P.out_hi, P, gi, S.vhi[c], 27);
-            // the global phase pulls this trailing word if a target leaves the
-            // inner tile (another tile may list it as global) or is global here
-            bool need_lo = P.lo_full;
-            const uint32_t tm = S.tm[c];
-            uint32_t out = 0;  // directions that leave the inner tile
-            if (lx == 0) out |= 0x64u;       // W NW SW
-            if (lx == TX - 1) out |= 0x91u;  // E NE SE
-            if (ly == 0) out |= 0x32u;       // N NE NW
-            if (ly == TY - 1) out |= 0xC8u;  // S SW SE
-            need_lo |= (tm & out) != 0;
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-                need_lo |= ((tm >> k) & 1u) && S.gf[c + offy(k) * EX + offx(k)];
-            if (need_lo) wr_f(P.out_lo, P, gi, S.vlo[c], 28);
+            const float2 a = S.v[ey * EX + ex];
+            wr_f(P.out_hi, P, gi, a.x, 27);
+            wr_f(P.out_lo, P, gi, a.y, 28);
         }
     }
-    for (int o = 16; o; o >>= 1) done += __shfl_down_sync(0xffffffffu, done, o);
-    if (tid == 0) S.done = 0;
+    done = __reduce_add_sync(0xffffffffu, done);
+    if (lane == 0 && done) atomicAdd(&S.ndone, done);
     __syncthreads();
-    if ((tid & 31) == 0 && done) atomicAdd(&S.done, done);
-    __syncthreads();
-    if (tid == 0) {
-        if (S.done) atomicAdd(&G->done_cells, S.done);
-        if (S.gave_up) atomicMax(&G->status, kStatusNoProgress);
-    }
+    if (tid == 0 && S.ndone) atomicAdd(&G->done_cells, (unsigned long long)S.ndone);
 }
 
 template <Mode M, bool BATCH>
 cudaError_t launch_local_halo(const Prob& P, EngineGlobals* G, const Prob* probs,
                               const int64_t* prefix, int nprob, int64_t tiles, cudaStream_t s) {
-    constexpr size_t sm = sizeof(SmemHalo);
+    constexpr size_t sm = sizeof(SmemHalo<HaloMode<M>::kMfd>);
     static std::atomic<unsigned long long> set_on{0};
     cudaError_t e = smem_limit_once(k_local_halo<M, BATCH>, sm, set_on);
     if (e != cudaSuccess) return e;
     if (tiles > 0)
-        k_local_halo<M, BATCH><<<(unsigned)tiles, kHaloNT, sm, s>>>(P, G, probs, prefix, nprob,
-                                                                  wait_limit_ns());
+        k_local_halo<M, BATCH><<<(unsigned)tiles, kHaloNT, sm, s>>>(P, G, probs, prefix, nprob);
     return cudaGetLastError();
 }
 
