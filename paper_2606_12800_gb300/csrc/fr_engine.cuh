@@ -433,6 +433,12 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 
+__device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
     unsigned v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -497,9 +503,11 @@ template <Mode M, bool W, bool AREA>
 __global__ void __launch_bounds__(256) k_global_levels(const Prob* __restrict__ probs, Prob single,
                                                        EngineGlobals* G,
                                                        unsigned long long total_cells,
+                                                       unsigned long long poll_max,
                                                        unsigned long long limit_ns) {
     using E = Eng<M, W, AREA>;
     __shared__ unsigned long long s_done;
+    if (__ldcg(&G->glist_count) <= poll_max) return;  // k_global_poll takes them
     const Prob& P0 = probs ? probs[0] : single;
     unsigned long long* const buf_a = reinterpret_cast<unsigned long long*>(P0.link);
     unsigned long long* const buf_b = P0.glist;
@@ -578,9 +586,174 @@ __global__ void __launch_bounds__(256) k_global_levels(const Prob* __restrict__ 
     }
 }
 
+// ---------------------------------------------------- polling global phase
+// The same cells when there are few of them (up to kPollCells per resident
+// lane), which is the rule on terrain: every lane owns its cells of the list
+// and reads the values of their dependencies until all are there.  The local
+// phase has put kPending into both words of every global cell, a NaN that no
+// sum yields, so a value is its own flag: a finished cell costs two stores and
+// the next one in the chain sees them at its next load, one trip to L2 per
+// link.  No counters, arrivals, fences or queues, each of which is a trip of
+// its own: with rounds and grid barriers a link took 10 to 20 us (17 links on
+// 777x1333 180 us, 27 on 2048^2 335 us, 30 on 8192^2 620 us), a queue of ready
+// cells between the lanes took as long (225, 390 and 520 us).
+//
+// A lane tries its cells in turn and never waits at one, and the launch is
+// cooperative (every lane runs), so an acyclic routing always gets on.  Where
+// nothing has been finished anywhere for kPollStuck tries (a cycle), or for the
+// wait limit, the lanes leave; the completion count reports the rest.
+constexpr int kPollCells = 4;
+constexpr int kPollStuck = 1 << 14;
+constexpr uint32_t kPending = 0xFFC0DEADu;
+
+__device__ __forceinline__ bool pending(float v) { return __float_as_uint(v) == kPending; }
+
+// Row and column of cell t (32-bit division where the grid allows it).
+__device__ __forceinline__ void cell_xy(const Prob& P, int64_t t, int64_t& x, int64_t& y) {
+    y = ((uint64_t)ncell(P) >> 32) ? t / P.nx : (int64_t)((uint32_t)t / (uint32_t)P.nx);
+    x = t - y * P.nx;
+}
+
+// Computes and publishes cell t if its dependencies are final.
+template <class E>
+__device__ __forceinline__ bool poll_step(const Prob& P, int64_t t) {
+    static_assert(E::kBranch, "modes with several targets per cell");
+    int64_t x, y;
+    cell_xy(P, t, x, y);
+    const uint32_t gm = grid_mask(x, y, P.nx, P.ny);
+    const uint32_t recv = g_recv<E>(P, t) & gm;
+    uint32_t dep = recv;
+    if constexpr (!E::kAdj) {
+        dep = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const uint8_t rb = ((gm >> k) & 1u) ? rd_rb(P, t + offi(k, P.nx)) : (uint8_t)0;
+            dep |= ((recv_mask<E::kMfd>(rb) >> opp(k)) & (gm >> k) & 1u) << k;
+        }
+    }
+    float f[8];
+    df vv[8];
+    bool ready = true;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        f[k] = 0.0f;
+        vv[k] = df_make(0.0f);
+        if (!((dep >> k) & 1u)) continue;
+        const int64_t j = t + offi(k, P.nx);
+        vv[k] = g_value<E>(P, j);
+        f[k] = 1.0f;
+        if constexpr (E::kMfd) f[k] = E::kAdj ? __ldg(P.frac + t * 8 + k) : __ldg(P.frac + j * 8 + opp(k));
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) ready &= !pending(vv[k].hi) && !pending(vv[k].lo);
+    if (!ready) return false;
+    const df v = df_dot8(init_value<E>(P, t, recv), f, vv);  // the fixed order
+    wr_f(P.out_hi, P, t, v.hi, 13);
+    wr_f(P.out_lo, P, t, v.lo, 14);
+    return true;
+}
+
+template <Mode M, bool W, bool AREA>
+__global__ void __launch_bounds__(256) k_global_poll(const Prob* __restrict__ probs, Prob single,
+                                                     EngineGlobals* G, unsigned long long total_cells,
+                                                     unsigned long long poll_max, unsigned long long limit_ns) {
+    using E = Eng<M, W, AREA>;
+    __shared__ unsigned long long s_done;
+    const unsigned long long count = __ldcg(&G->glist_count);
+    if (count > poll_max) return;  // the rounds take them
+    const Prob& P0 = probs ? probs[0] : single;
+    constexpr unsigned long long kCellMask = (1ull << 40) - 1;
+    const unsigned long long lanes = (unsigned long long)gridDim.x * blockDim.x;
+    // Neighbours in the list are mostly neighbours on the ground and share cache
+    // lines, so a block takes consecutive cells; where that would leave most SMs
+    // without work, a warp does and the warps spread over the blocks.  Measured
+    // (blocks / warps / single cells spread): 403 K cells on 155 K lanes 238 /
+    // 305 / 441 us, 25 K cells 63 / 55 / 55 us, 3.5 K cells 54 / 36 / 34 us.
+    const unsigned long long me =
+        count > lanes / 2 ? (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x
+                          : ((unsigned long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
+    unsigned todo = 0;
+#pragma unroll
+    for (int j = 0; j < kPollCells; ++j) todo |= (unsigned)(me + j * lanes < count) << j;
+    unsigned done = 0, stuck = 0;
+    unsigned long long seen = ~0ull, since = 0;
+    while (__any_sync(0xffffffffu, todo != 0)) {
+        unsigned got = 0;
+#pragma unroll 1
+        for (int j = 0; j < kPollCells; ++j) {
+            if (!((todo >> j) & 1u)) continue;
+            const unsigned long long item = __ldg(P0.glist + me + j * lanes);
+            const Prob& P = probs ? probs[(int)(item >> 40)] : single;
+            if (poll_step<E>(P, (int64_t)(item & kCellMask))) {
+                todo &= ~(1u << j);
+                ++got;
+            }
+        }
+        done += got;
+        const unsigned n = __reduce_add_sync(0xffffffffu, got);
+        if (n) {
+            if ((threadIdx.x & 31) == 0) atomicAdd(&G->rounds, (unsigned long long)n);  // cells finished so far
+            stuck = 0;
+            continue;
+        }
+        // nothing here this time: has anything been finished elsewhere?
+        int stop = 0;
+        if ((threadIdx.x & 31) == 0) {
+            if ((stuck & 63u) == 0) {
+                const unsigned long long now = global_ns(), all = ld_relaxed_u64(&G->rounds);
+                if (all != seen) {
+                    seen = all;
+                    since = now;
+                    stuck = 0;
+                }
+                if (now - since >= limit_ns) stop = 2;
+            }
+            if (++stuck > kPollStuck) stop = 1;
+            if (stop == 2) atomicMax(&G->status, kStatusNoProgress);
+        }
+        if (__shfl_sync(0xffffffffu, stop, 0)) break;
+    }
+    done = __reduce_add_sync(0xffffffffu, done);
+    if (threadIdx.x == 0) s_done = 0;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0 && done) atomicAdd(&s_done, (unsigned long long)done);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (s_done) atomicAdd(&G->done_cells, s_done);
+        __threadfence();
+        const unsigned fin = atomicAdd(&G->finished_ctas, 1u);
+        if (fin == gridDim.x - 1) {
+            __threadfence();
+            const unsigned long long got = atomicAdd(&G->done_cells, 0ull);
+            if (got != total_cells) atomicMax(&G->status, kStatusNoProgress);
+        }
+    }
+}
+
+// Blocks of a cooperative launch of `kernel` on the current device: at most
+// per_sm per SM; kept per device.
+template <class K>
+cudaError_t coop_grid(K kernel, int per_sm, int (&grid_of)[64], int& grid) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    grid = dev < 64 ? grid_of[dev] : 0;
+    if (grid) return cudaSuccess;
+    int sms = 0, per = 0;
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, 256, 0);
+    if (e != cudaSuccess) return e;
+    if (per < 1) return cudaErrorInvalidConfiguration;
+    grid = sms * (per < per_sm ? per : per_sm);
+    if (dev < 64) grid_of[dev] = grid;
+    return cudaSuccess;
+}
+
 // Launches the global phase: D8 forward keeps the single-successor walkers
-// (a D8 cell has one receiver, so nothing diverges); every other mode runs
-// the level-synchronous kernel as a cooperative launch.
+// (a D8 cell has one receiver, so nothing diverges); every other mode polls, or
+// runs the level-synchronous kernel if there are many global cells (both are
+// cooperative launches; the one not chosen returns at once).
 template <Mode M, bool W, bool AREA>
 cudaError_t launch_global(const Prob* probs, const Prob& single, EngineGlobals* G,
                           unsigned long long total_cells, cudaStream_t s) {
@@ -591,31 +764,24 @@ cudaError_t launch_global(const Prob* probs, const Prob& single, EngineGlobals* 
         k_global<M, W, AREA><<<walker_grid(), 256, 0, s>>>(probs, single, G, total_cells);
         return cudaGetLastError();
     } else {
-        static int grid_of[64] = {};
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
+        static int grid_poll[64] = {}, grid_lev[64] = {};
+        int gp = 0, gl = 0;
+        cudaError_t e = coop_grid(k_global_poll<M, W, AREA>, 4, grid_poll, gp);
         if (e != cudaSuccess) return e;
-        int grid = dev < 64 ? grid_of[dev] : 0;
-        if (grid == 0) {
-            int sms = 0, per = 0;
-            e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            if (e != cudaSuccess) return e;
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_global_levels<M, W, AREA>, 256, 0);
-            if (e != cudaSuccess) return e;
-            if (per < 1) return cudaErrorInvalidConfiguration;
-            // one block per SM: a round's frontier (about 20 K cells on an 8192^2
-            // slope-split route) fits, and the grid barrier has the fewest
-            // arrivals (measured faster than two or four blocks per SM)
-            grid = sms;
-            if (dev < 64) grid_of[dev] = grid;
-        }
+        // one block per SM: a round's frontier (about 20 K cells on an 8192^2
+        // slope-split route) fits, and the grid barrier has the fewest
+        // arrivals (measured faster than two or four blocks per SM)
+        e = coop_grid(k_global_levels<M, W, AREA>, 1, grid_lev, gl);
+        if (e != cudaSuccess) return e;
         Prob one = single;
         const Prob* pp = probs;
         unsigned long long total = total_cells;
+        unsigned long long poll_max = (unsigned long long)gp * 256 * kPollCells;
         unsigned long long limit = wait_limit_ns();
-        void* args[] = {(void*)&pp, (void*)&one, (void*)&G, (void*)&total, (void*)&limit};
-        return cudaLaunchCooperativeKernel((const void*)k_global_levels<M, W, AREA>, dim3(grid),
-                                           dim3(256), args, 0, s);
+        void* args[] = {(void*)&pp, (void*)&one, (void*)&G, (void*)&total, (void*)&poll_max, (void*)&limit};
+        e = cudaLaunchCooperativeKernel((const void*)k_global_poll<M, W, AREA>, dim3(gp), dim3(256), args, 0, s);
+        if (e != cudaSuccess) return e;
+        return cudaLaunchCooperativeKernel((const void*)k_global_levels<M, W, AREA>, dim3(gl), dim3(256), args, 0, s);
     }
 }
 

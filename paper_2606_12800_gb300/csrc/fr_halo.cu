@@ -137,8 +137,8 @@ __device__ __forceinline__ bool bar_or(int id, int n, bool p) {
 }
 
 // Marks the global inner cells of a warp (all 32 lanes call; glob: this
-// lane's cell gi is global): their bits, and list entries reserved with one
-// atomic per warp.
+// lane's cell gi is global): their bits, list entries reserved with one
+// atomic per warp, and their values pending (see k_global_poll).
 __device__ __forceinline__ void mark_global_cells(const Prob& P, EngineGlobals* G, int64_t gi,
                                                   int pid, bool glob) {
     const unsigned m = __ballot_sync(0xffffffffu, glob);
@@ -152,6 +152,8 @@ __device__ __forceinline__ void mark_global_cells(const Prob& P, EngineGlobals* 
         const unsigned long long slot = base + __popc(m & ((1u << lane) - 1u));
         if (FR_OK((int64_t)slot, P.glist_cap, 17))
             P.glist[slot] = ((unsigned long long)pid << 40) | (unsigned long long)gi;
+        wr_f(P.out_hi, P, gi, __uint_as_float(kPending), 27);
+        wr_f(P.out_lo, P, gi, __uint_as_float(kPending), 28);
     }
 }
 
@@ -616,12 +618,12 @@ cudaError_t launch_halo_single(const Prob& P, EngineGlobals* G, cudaStream_t s) 
 
 }  // namespace
 
-// MFD forward accumulation: halo-tile local phase + level-synchronous global phase.
+// MFD forward accumulation: halo-tile local phase + global phase.
 cudaError_t launch_mfd_forward(const Prob& P, EngineGlobals* G, cudaStream_t s) {
     return launch_halo_single<Mode::FwdMfd>(P, G, s);
 }
 
-// Adjoint (D8 or MFD): halo-tile local phase + level-synchronous global phase.
+// Adjoint (D8 or MFD): halo-tile local phase + global phase.
 cudaError_t launch_adjoint(bool mfd, const Prob& P, EngineGlobals* G, cudaStream_t s) {
     return mfd ? launch_halo_single<Mode::AdjMfd>(P, G, s) : launch_halo_single<Mode::AdjD8>(P, G, s);
 }
