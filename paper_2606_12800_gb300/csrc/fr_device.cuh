@@ -70,15 +70,6 @@ __device__ __forceinline__ df df_mul(df a, df b) {
     return df_norm(p, e);
 }
 
-// Sum of eight two-float terms in a fixed pairwise order:
-// ((t0 + t1) + (t2 + t3)) + ((t4 + t5) + (t6 + t7)).  Absent terms are zero,
-// which df_add passes through exactly (the MFD normaliser S uses this order).
-__device__ __forceinline__ df df_tree8(const df (&t)[8]) {
-    const df a = df_add(df_add(t[0], t[1]), df_add(t[2], t[3]));
-    const df b = df_add(df_add(t[4], t[5]), df_add(t[6], t[7]));
-    return df_add(a, b);
-}
-
 // own + sum over k = 0..7 of f[k] * v[k], accumulated in ascending k with
 // compensation (the Dot2 scheme of Ogita, Rump and Oishi, 2005, with two-float
 // v): each product is split exactly by an FMA, each partial sum by Knuth's
@@ -174,40 +165,38 @@ __host__ __device__ inline MfdConst make_mfd_const(double dx, double p) {
     return m;
 }
 
-// s^p for a positive normal s: s^pn (repeated products) times 2^(pf log2 s).
-// log2 s = e + log2(m) from the exponent e and a mantissa m in [1/sqrt2, sqrt2]
-// (hardware log2, absolute error at most 2^-22 there); pf * e is kept exact as
-// a two-float (FMA); the power of two is split into an integer k and a rest
-// |x| <= ln2/2, and e^x is summed as its Taylor series to degree 7 (truncation
-// below 6e-9).  Relative error about 1e-7 for p in [1, 2], independent of the
-// magnitude of s.  Other s (zero, subnormal, infinite, NaN) fall back to powf.
-__device__ __forceinline__ float mfd_pow(float s, const MfdConst& c) {
-    if (!(s >= 1.17549435e-38f && s <= 3.0e38f)) return powf(s, c.p);
+// s^p for a positive s in the normal range: s^pn (repeated products) times
+// 2^(pf log2 s).  log2 s = e + log2(m) from the exponent e and a mantissa m in
+// [1/sqrt2, sqrt2) (hardware log2, absolute error at most 2^-22 there); pf * e
+// is kept exact as a two-float (FMA); the power of two is split into an integer
+// k and a rest |r| <= 1/2, and 2^r = 1 + r g(r) with g the polynomial that
+// interpolates (2^r - 1) / r at the seven Chebyshev points of [-0.502, 0.502]
+// (relative error of 2^r 2.4e-9, 1 at r = 0 exactly).  Integers come and go
+// through the low bits of floats near 2^23 * 1.5, not through the conversion
+// unit.  Relative error about 1e-7 for p in [1, 2], independent of the
+// magnitude of s.
+__device__ __forceinline__ float mfd_pow_normal(float s, const MfdConst& c) {
+    constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23: adding it rounds to an integer in the low bits
     const int bits = __float_as_int(s);
-    int e = ((bits >> 23) & 0xFF) - 127;
-    float m = __int_as_float((bits & 0x007FFFFF) | 0x3F800000);
-    if (m > 1.41421356f) {
-        m = __fmul_rn(m, 0.5f);
-        e += 1;
-    }
-    const float fe = (float)e;
+    const int tb = bits - 0x3F3504F3;  // exponent field relative to 1/sqrt2
+    const float m = __int_as_float(bits - (tb & (int)0xFF800000));
+    const float fe = __fsub_rn(__int_as_float((tb >> 23) + 0x4B400000), kMagic);
+    float lg;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg) : "f"(m));
     const float a = __fmul_rn(c.pf, fe);
     const float ae = __fmaf_rn(c.pf, fe, -a);
-    const float b = __fmul_rn(c.pf, __log2f(m));
-    float k = rintf(a);
-    float r = __fadd_rn(__fadd_rn(__fsub_rn(a, k), b), ae);
-    const float k2 = rintf(r);
-    r = __fsub_rn(r, k2);
-    k = __fadd_rn(k, k2);
-    const float x = __fmul_rn(r, 0.693147180559945309f);
-    float q = __fmaf_rn(x, 1.0f / 5040.0f, 1.0f / 720.0f);
-    q = __fmaf_rn(x, q, 1.0f / 120.0f);
-    q = __fmaf_rn(x, q, 1.0f / 24.0f);
-    q = __fmaf_rn(x, q, 1.0f / 6.0f);
-    q = __fmaf_rn(x, q, 0.5f);
-    q = __fmaf_rn(x, q, 1.0f);
-    q = __fmaf_rn(x, q, 1.0f);
-    float y = __fmul_rn(q, __int_as_float(((int)k + 127) << 23));
+    const float b = __fmul_rn(c.pf, lg);
+    const float km = __fadd_rn(__fadd_rn(a, b), kMagic);
+    const float r = __fadd_rn(__fadd_rn(__fsub_rn(a, __fsub_rn(km, kMagic)), b), ae);
+    float q = __fmaf_rn(r, 1.5297681e-05f, 1.5461909e-04f);
+    q = __fmaf_rn(r, q, 1.3333502e-03f);
+    q = __fmaf_rn(r, q, 9.6180551e-03f);
+    q = __fmaf_rn(r, q, 5.5504110e-02f);
+    q = __fmaf_rn(r, q, 2.4022651e-01f);
+    q = __fmaf_rn(r, q, 6.9314718e-01f);
+    q = __fmaf_rn(r, q, 1.0f);
+    float y = __int_as_float(__float_as_int(q) + (__float_as_int(km) << 23));  // times 2^k
+    if (c.pn == 1) return __fmul_rn(y, s);
 #pragma unroll 1
     for (int i = 0; i < c.pn; ++i) y = __fmul_rn(y, s);
     return y;
@@ -216,8 +205,9 @@ __device__ __forceinline__ float mfd_pow(float s, const MfdConst& c) {
 // u_k = s_k^p for a strictly lower neighbour, s_k = (zc - zn)/d_k.  The drop
 // and the product with 1/d are carried as two-float and the trailing word is
 // applied as a first-order correction of the power: (s+e)^p ~ s^p (1 + p e/s)
-// (the quotient e/s only scales a correction of relative size 1e-7, so a
-// fast division suffices).
+// (the quotient e/s only scales a correction of relative size 1e-7, so an
+// approximate reciprocal suffices).  Slopes outside the normal range (zero,
+// subnormal, huge, infinite, NaN) fall back to powf.
 __device__ __forceinline__ float mfd_u(float zc, float zn, int k, const MfdConst& m) {
     float dz = __fsub_rn(zc, zn);
     float bb = __fsub_rn(dz, zc);
@@ -228,14 +218,15 @@ __device__ __forceinline__ float mfd_u(float zc, float zn, int k, const MfdConst
     float se = __fmaf_rn(dz, ch, -s);
     se = __fmaf_rn(dz, cl, se);
     se = __fmaf_rn(dze, ch, se);
-    float u = mfd_pow(s, m);
-    float corr = __fmul_rn(m.p, __fdividef(se, s));
-    return __fmaf_rn(u, corr, u);
-}
-
-// Out-of-line copy of mfd_u for loops that would otherwise replicate powf.
-static __device__ __noinline__ float mfd_u_call(float zc, float zn, int k, MfdConst m) {
-    return mfd_u(zc, zn, k, m);
+    // s in [2^-126, 2^126): one comparison of the bits
+    if ((unsigned)(__float_as_int(s) - 0x00800000) < 0x7E000000u) {
+        float rs;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rs) : "f"(s));
+        const float u = mfd_pow_normal(s, m);
+        return __fmaf_rn(u, __fmul_rn(m.p, __fmul_rn(se, rs)), u);
+    }
+    const float u = powf(s, m.p);
+    return __fmaf_rn(u, __fmul_rn(m.p, __fdividef(se, s)), u);
 }
 
 // Two-float reciprocal of the normaliser S = sum of u_k.
@@ -259,22 +250,29 @@ __device__ __forceinline__ uint32_t zero_bytes(uint32_t x) {
     return ~(((x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | x) & 0x80808080u;
 }
 
-// The fractions of a cell with receiver mask m (App. A): f_k = u_k / S with
-// S = sum of u_k over the mask, summed in the pairwise order of df_tree8 and
-// inverted as two-float, each f_k rounded once to fp32; 0 where bit k is clear.
-// Every MFD kernel takes its fractions from this one definition.
+// Fractions f_k = u_k / S from the weights u_k of a cell's receivers (0
+// elsewhere), with S the sum of the u_k in a fixed pairwise order
+// (((u0 + u1) + (u2 + u3)) + ((u4 + u5) + (u6 + u7)), two-float), inverted as two-float, and each f_k rounded once to fp32; 0 where bit k of m
+// is clear.  Every MFD kernel takes its fractions from this one definition.
+__device__ __forceinline__ void mfd_fracs_of(const float (&u)[8], uint32_t m, float (&f)[8]) {
+    df t[4];  // the tree's first sums: two floats add up exactly
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float a = u[2 * i], b = u[2 * i + 1], s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+        t[i] = {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+    }
+    const df inv = m ? df_recip(df_add(df_add(t[0], t[1]), df_add(t[2], t[3]))) : df_make(0.0f);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) f[k] = ((m >> k) & 1u) ? mfd_frac(u[k], inv).hi : 0.0f;
+}
+
+// The fractions of a cell with receiver mask m from the elevations around it.
 __device__ __forceinline__ void mfd_fracs8(float zc, const float (&zn)[8], uint32_t m,
                                            const MfdConst& mc, float (&f)[8]) {
     float u[8];
-    df t[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        u[k] = ((m >> k) & 1u) ? mfd_u(zc, zn[k], k, mc) : 0.0f;
-        t[k] = df_make(u[k]);
-    }
-    const df inv = m ? df_recip(df_tree8(t)) : df_make(0.0f);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) f[k] = ((m >> k) & 1u) ? mfd_frac(u[k], inv).hi : 0.0f;
+    for (int k = 0; k < 8; ++k) u[k] = ((m >> k) & 1u) ? mfd_u(zc, zn[k], k, mc) : 0.0f;
+    mfd_fracs_of(u, m, f);
 }
 
 // D-infinity (Tarboton) receivers and fractions of one cell: the steepest of

@@ -109,6 +109,25 @@ def _check(ny, nx, make, flags, with_rain):
     np.testing.assert_array_equal(g.cpu().numpy(), _solve(mask, frac, gbar, adjoint=True)[0])
 
 
+@pytest.mark.parametrize("shape", [(15, 63), (16, 64), (17, 65), (18, 66), (33, 129), (1, 70), (70, 1), (2, 2)])
+@pytest.mark.parametrize("flags", [0, oracle.EDGE_ROUTE])
+@pytest.mark.parametrize("p", [0.5, 1.0, 1.1, 4.5])
+def test_mfd_weights_tile_edges(shape, flags, p):
+    """Masks (with and without fractions) bit for bit, fractions against FP64 at
+    the edges of the 64x16 tiles.  A fraction's error: the powers' 1e-7 (p 4.5:
+    the slope's rounding times p) twice, and its own rounding."""
+    from paper_2606_12800_gb300 import api
+    z = inputs.fractal_dem(*shape, beta=2.0, tilt=0.0, seed=6)
+    zt = torch.from_numpy(z).cuda()
+    m_ref, f_ref = oracle.receivers_mfd(z, 30.0, p, flags)
+    m, f = api.receivers_mfd(zt, 30.0, p, flags, frac=True)
+    np.testing.assert_array_equal(m.cpu().numpy(), m_ref)
+    np.testing.assert_array_equal(api.receivers_mfd(zt, 30.0, p, flags).cpu().numpy(), m_ref)
+    f = f.cpu().numpy().astype(np.float64).reshape(-1, 8)
+    f_ref = f_ref.reshape(-1, 8)
+    assert np.all(np.abs(f - f_ref) <= 1e-6 * f_ref)
+
+
 @pytest.mark.parametrize("shape", [(64, 80), (63, 79), (65, 81), (128, 160), (129, 161), (3, 250), (250, 3), (1, 96)])
 @pytest.mark.parametrize("make", [_rough, _ramp])
 @pytest.mark.parametrize("flags", [0, oracle.EDGE_ROUTE])
