@@ -128,6 +128,40 @@ def test_mfd_weights_tile_edges(shape, flags, p):
     assert np.all(np.abs(f - f_ref) <= 1e-6 * f_ref)
 
 
+@pytest.mark.parametrize("shape", [(15, 63), (16, 64), (17, 65), (33, 129), (3, 70), (70, 3), (2, 2)])
+@pytest.mark.parametrize("flags", [0, oracle.EDGE_ROUTE])
+def test_mfd_grad_z_tile_edges(shape, flags):
+    """dL/dz against its formula in FP64 on the library's fractions and adjoint,
+    at the edges of the 64x16 tiles.  Per edge: the adjoint's leading words are
+    rounded (2^-24 each), six fp32 operations follow."""
+    from paper_2606_12800_gb300 import api
+    ny, nx = shape
+    z = inputs.fractal_dem(ny, nx, beta=2.0, tilt=0.0, seed=8)
+    zt = torch.from_numpy(z).cuda()
+    out = api.route_mfd(zt, 30.0, 1.1, None, flags, want_lo=True, want_mask=True)
+    gbar = torch.from_numpy(inputs.rain_field(ny, nx, 4)).cuda()
+    R = api.routing_mfd(out["mask"], zt, 30.0, 1.1, flags)
+    g, dz = api.adjoint(R, out["w"], out["w_lo"], dLdw=gbar, want_dz=True)
+    _, f = api.receivers_mfd(zt, 30.0, 1.1, flags, frac=True)
+    f = f.cpu().numpy().astype(np.float64)
+    g, w = g.double().cpu().numpy(), out["w"].double().cpu().numpy()
+    z = z.astype(np.float64)
+    ref, tol = np.zeros((ny, nx)), np.full((ny, nx), 1e-30)
+    for y in range(ny):
+        for x in range(nx):
+            on = [k for k in range(8) if f[y, x, k] > 0]
+            G = sum(f[y, x, k] * g[y + OFF[k][1], x + OFF[k][0]] for k in on)
+            for k in on:
+                yn, xn = y + OFF[k][1], x + OFF[k][0]
+                c = 1.1 * w[y, x] * f[y, x, k] / (z[y, x] - z[yn, xn])
+                a, e = c * (g[yn, xn] - G), c * (g[yn, xn] + G) * 8 * 2.0 ** -24
+                ref[y, x] += a
+                ref[yn, xn] -= a
+                tol[y, x] += e
+                tol[yn, xn] += e
+    assert np.all(np.abs(dz.double().cpu().numpy() - ref) <= tol)
+
+
 @pytest.mark.parametrize("shape", [(64, 80), (63, 79), (65, 81), (128, 160), (129, 161), (3, 250), (250, 3), (1, 96)])
 @pytest.mark.parametrize("make", [_rough, _ramp])
 @pytest.mark.parametrize("flags", [0, oracle.EDGE_ROUTE])
