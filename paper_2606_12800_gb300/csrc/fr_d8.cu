@@ -170,8 +170,8 @@ __device__ __forceinline__ void cp_async_wait_all() {
 
 // Lists the block's unfinished inner cells (local indices in S.queue, S.nglob
 // of them) as global: one list allocation per block, their bits or-ed once
-// per word and warp.  Called by all threads after a barrier.
-template <class S_>
+// per word and warp, their values pending (see k_global_poll).  Called by all threads after a barrier.
+template <bool W, bool AREA, class S_>
 __device__ __forceinline__ void list_global(S_& S, const Prob& P, EngineGlobals* G, int pid,
                                             int tx_inner, int64_t x0, int64_t y0, int nthreads) {
     const int ng = S.nglob;
@@ -187,6 +187,11 @@ __device__ __forceinline__ void list_global(S_& S, const Prob& P, EngineGlobals*
             gi = (y0 + ly) * P.nx + x0 + lx;
             if (FR_OK((int64_t)(base + i), P.glist_cap, 17))
                 P.glist[base + i] = ((unsigned long long)pid << 40) | (unsigned long long)gi;
+            if constexpr (W) {
+                wr_f(P.out_hi, P, gi, __uint_as_float(kPending), 27);
+                wr_f(P.out_lo, P, gi, __uint_as_float(kPending), 28);
+            }
+            if constexpr (AREA) wr_area(P, gi, kPendingArea);
         }
         // lanes whose cells share a word of bits or them together; one atomic per word
         const long long word = gi >= 0 ? (long long)(gi >> 5) : -1ll;
@@ -560,7 +565,7 @@ __global__ void __launch_bounds__(Gm::NT) k_local_d8(Prob Pone, EngineGlobals* G
         if (d) atomicAdd(&G->done_cells, d);
         if (AREA && !BATCH && S.sinks) atomicAdd(&G->sink_area, (unsigned long long)S.sinks);
     }
-    if (S.nglob) list_global(S, P, G, pid, TX, x0, y0, NT8);
+    if (S.nglob) list_global<W, AREA>(S, P, G, pid, TX, x0, y0, NT8);
 }
 
 template <class Gm, bool W, bool AREA, bool BATCH>

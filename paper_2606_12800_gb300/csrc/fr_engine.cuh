@@ -346,11 +346,12 @@ __device__ __forceinline__ void frontier_push(int64_t nx, int64_t cell, unsigned
 // frontier buffer).
 template <Mode M, bool W, bool AREA>
 __global__ void __launch_bounds__(256) k_global_init(const Prob* __restrict__ probs, Prob single,
-                                                     EngineGlobals* G) {
+                                                     EngineGlobals* G, unsigned long long poll_max) {
     using E = Eng<M, W, AREA>;
     const unsigned long long count = G->glist_count;
     const Prob& P0 = probs ? probs[0] : single;
-    if (count >= P0.skel_min) return;  // the skeleton solve takes the global cells
+    // the skeleton solve or the polling kernel takes the global cells
+    if (count >= P0.skel_min || count <= poll_max) return;
     const unsigned long long* list = P0.glist;
     unsigned long long* starts = reinterpret_cast<unsigned long long*>(P0.link);
     constexpr unsigned long long kCellMask = (1ull << 40) - 1;
@@ -378,12 +379,14 @@ __global__ void __launch_bounds__(256) k_global_init(const Prob* __restrict__ pr
 // that every cell of every problem was computed.
 template <Mode M, bool W, bool AREA>
 __global__ void __launch_bounds__(256) k_global(const Prob* __restrict__ probs, Prob single,
-                                                EngineGlobals* G, unsigned long long total_cells) {
+                                                EngineGlobals* G, unsigned long long total_cells,
+                                                unsigned long long poll_max) {
     using E = Eng<M, W, AREA>;
     static_assert(E::kD8Fwd, "branching modes use k_global_levels");
     __shared__ unsigned long long s_done;
     const Prob& P0 = probs ? probs[0] : single;
-    if (__ldcg(&G->glist_count) >= P0.skel_min) return;  // the skeleton solve takes them
+    const unsigned long long all = __ldcg(&G->glist_count);
+    if (all >= P0.skel_min || all <= poll_max) return;  // the skeleton solve or the polling kernel takes them
     const unsigned long long count = G->fcount[0];
     const unsigned long long* starts = reinterpret_cast<const unsigned long long*>(P0.link);
     unsigned long long done = 0;
@@ -596,7 +599,10 @@ __global__ void __launch_bounds__(256) k_global_levels(const Prob* __restrict__ 
 // link.  No counters, arrivals, fences or queues, each of which is a trip of
 // its own: with rounds and grid barriers a link took 10 to 20 us (17 links on
 // 777x1333 180 us, 27 on 2048^2 335 us, 30 on 8192^2 620 us), a queue of ready
-// cells between the lanes took as long (225, 390 and 520 us).
+// cells between the lanes took as long (225, 390 and 520 us).  For D8 forward
+// the walkers (a counter preset per cell, then steps of loads, fence and
+// arrival) took 41 us on 160x192, 56 on 1537x2603 and 57 on 4096^2, polling 17,
+// 25 and 23 us.
 //
 // A lane tries its cells in turn and never waits at one, and the launch is
 // cooperative (every lane runs), so an acyclic routing always gets on.  Where
@@ -605,6 +611,7 @@ __global__ void __launch_bounds__(256) k_global_levels(const Prob* __restrict__ 
 constexpr int kPollCells = 4;
 constexpr int kPollStuck = 1 << 14;
 constexpr uint32_t kPending = 0xFFC0DEADu;
+constexpr uint64_t kPendingArea = ~0ull;  // areas: above any count of cells
 
 __device__ __forceinline__ bool pending(float v) { return __float_as_uint(v) == kPending; }
 
@@ -614,10 +621,57 @@ __device__ __forceinline__ void cell_xy(const Prob& P, int64_t t, int64_t& x, in
     x = t - y * P.nx;
 }
 
+// The same for D8 forward routing (water in ascending code order, areas): the
+// walkers' sums.
+template <class E>
+__device__ __forceinline__ bool poll_step_d8(const Prob& P, int64_t t) {
+    int64_t x, y;
+    cell_xy(P, t, x, y);
+    const uint32_t gm = grid_mask(x, y, P.nx, P.ny);
+    uint32_t don = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        if ((gm >> k) & 1u) don |= (uint32_t)(rd_rb(P, t + offi(k, P.nx)) == (uint8_t)opp(k)) << k;
+    bool ready = true;
+    df vv[8];
+    uint64_t a[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int64_t j = t + offi(k, P.nx);
+        const bool on = (don >> k) & 1u;
+        vv[k] = df_make(0.0f);
+        a[k] = 0;
+        if constexpr (E::kVal) {
+            if (on) vv[k] = g_value<E>(P, j);
+        }
+        if constexpr (E::kArea) {
+            if (on) a[k] = rd_area(P, j);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) ready &= !pending(vv[k].hi) && !pending(vv[k].lo) && a[k] != kPendingArea;
+    if (!ready) return false;
+    if constexpr (E::kVal) {
+        df v = init_value<E>(P, t, 0u);
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if ((don >> k) & 1u) v = df_add(v, vv[k]);
+        wr_f(P.out_hi, P, t, v.hi, 13);
+        wr_f(P.out_lo, P, t, v.lo, 14);
+    }
+    if constexpr (E::kArea) {
+        uint64_t s = 1;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s += a[k];
+        wr_area(P, t, s);
+    }
+    return true;
+}
+
 // Computes and publishes cell t if its dependencies are final.
 template <class E>
 __device__ __forceinline__ bool poll_step(const Prob& P, int64_t t) {
-    static_assert(E::kBranch, "modes with several targets per cell");
+    if constexpr (E::kD8Fwd) return poll_step_d8<E>(P, t);
     int64_t x, y;
     cell_xy(P, t, x, y);
     const uint32_t gm = grid_mask(x, y, P.nx, P.ny);
@@ -660,8 +714,9 @@ __global__ void __launch_bounds__(256) k_global_poll(const Prob* __restrict__ pr
     using E = Eng<M, W, AREA>;
     __shared__ unsigned long long s_done;
     const unsigned long long count = __ldcg(&G->glist_count);
-    if (count > poll_max) return;  // the rounds take them
     const Prob& P0 = probs ? probs[0] : single;
+    // the rounds (D8 forward: the walkers or the skeleton) take them
+    if (count > poll_max || (E::kD8Fwd && count >= P0.skel_min)) return;
     constexpr unsigned long long kCellMask = (1ull << 40) - 1;
     const unsigned long long lanes = (unsigned long long)gridDim.x * blockDim.x;
     // Neighbours in the list are mostly neighbours on the ground and share cache
@@ -750,36 +805,40 @@ cudaError_t coop_grid(K kernel, int per_sm, int (&grid_of)[64], int& grid) {
     return cudaSuccess;
 }
 
-// Launches the global phase: D8 forward keeps the single-successor walkers
-// (a D8 cell has one receiver, so nothing diverges); every other mode polls, or
-// runs the level-synchronous kernel if there are many global cells (both are
-// cooperative launches; the one not chosen returns at once).
+// Launches the global phase: the polling kernel, and behind it what takes more
+// global cells than it can: for D8 forward the single-successor walkers (a D8
+// cell has one receiver, so nothing diverges), else the level-synchronous kernel.
+// Polling and levels are cooperative launches; a kernel whose turn it is not
+// returns at once, and one whose turn cannot come for a grid of this size is not
+// launched.
 template <Mode M, bool W, bool AREA>
 cudaError_t launch_global(const Prob* probs, const Prob& single, EngineGlobals* G,
                           unsigned long long total_cells, cudaStream_t s) {
+    static int grid_poll[64] = {};
+    int gp = 0;
+    cudaError_t e = coop_grid(k_global_poll<M, W, AREA>, 4, grid_poll, gp);
+    if (e != cudaSuccess) return e;
+    Prob one = single;
+    const Prob* pp = probs;
+    unsigned long long total = total_cells;
+    unsigned long long poll_max = (unsigned long long)gp * 256 * kPollCells;
+    unsigned long long limit = wait_limit_ns();
+    void* args[] = {(void*)&pp, (void*)&one, (void*)&G, (void*)&total, (void*)&poll_max, (void*)&limit};
+    e = cudaLaunchCooperativeKernel((const void*)k_global_poll<M, W, AREA>, dim3(gp), dim3(256), args, 0, s);
+    if (e != cudaSuccess || total_cells <= poll_max) return e;
     if constexpr (M == Mode::FwdD8) {
-        k_global_init<M, W, AREA><<<walker_grid(), 256, 0, s>>>(probs, single, G);
-        cudaError_t e = cudaGetLastError();
+        k_global_init<M, W, AREA><<<walker_grid(), 256, 0, s>>>(probs, single, G, poll_max);
+        e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        k_global<M, W, AREA><<<walker_grid(), 256, 0, s>>>(probs, single, G, total_cells);
+        k_global<M, W, AREA><<<walker_grid(), 256, 0, s>>>(probs, single, G, total_cells, poll_max);
         return cudaGetLastError();
     } else {
-        static int grid_poll[64] = {}, grid_lev[64] = {};
-        int gp = 0, gl = 0;
-        cudaError_t e = coop_grid(k_global_poll<M, W, AREA>, 4, grid_poll, gp);
-        if (e != cudaSuccess) return e;
+        static int grid_lev[64] = {};
+        int gl = 0;
         // one block per SM: a round's frontier (about 20 K cells on an 8192^2
         // slope-split route) fits, and the grid barrier has the fewest
         // arrivals (measured faster than two or four blocks per SM)
         e = coop_grid(k_global_levels<M, W, AREA>, 1, grid_lev, gl);
-        if (e != cudaSuccess) return e;
-        Prob one = single;
-        const Prob* pp = probs;
-        unsigned long long total = total_cells;
-        unsigned long long poll_max = (unsigned long long)gp * 256 * kPollCells;
-        unsigned long long limit = wait_limit_ns();
-        void* args[] = {(void*)&pp, (void*)&one, (void*)&G, (void*)&total, (void*)&poll_max, (void*)&limit};
-        e = cudaLaunchCooperativeKernel((const void*)k_global_poll<M, W, AREA>, dim3(gp), dim3(256), args, 0, s);
         if (e != cudaSuccess) return e;
         return cudaLaunchCooperativeKernel((const void*)k_global_levels<M, W, AREA>, dim3(gl), dim3(256), args, 0, s);
     }
