@@ -128,7 +128,8 @@ bool routing_ok(const fr_routing* R) {
     return false;
 }
 
-Prob base_prob(const fr_routing* R, char* ws) {
+// with_water: the D8 accumulation solves water (the skeleton's tile size).
+Prob base_prob(const fr_routing* R, char* ws, bool with_water = false) {
     Layout L = layout(R->nx * R->ny);
     Prob P;
     std::memset(&P, 0, sizeof(P));
@@ -147,10 +148,11 @@ Prob base_prob(const fr_routing* R, char* ws) {
     // starts, dependency slots
     P.skel_min = ~0ull;
     if (R->kind == FR_ROUTING_D8) {
-        const int64_t n = R->nx * R->ny, st = skel_tiles(R->nx, R->ny);
+        const int side = skel_side(with_water);
+        const int64_t n = R->nx * R->ny, st = skel_tiles(R->nx, R->ny, side);
         const size_t o_starts = align256((size_t)st * 4);
-        const size_t o_pool = o_starts + align256((size_t)st * (4 * kSkelTile - 4) * 8);
-        const size_t need = o_pool + (size_t)st * kSkelPool * 2;
+        const size_t o_pool = o_starts + align256((size_t)st * (4 * side - 4) * 8);
+        const size_t need = o_pool + (size_t)st * skel_pool(side) * 2;
         if (need <= (size_t)n * 8 && !(R->flags & FR_GLOBAL_WALKERS)) {
             char* base = ws + L.glist;
             P.sktiles = reinterpret_cast<uint32_t*>(base);
@@ -280,7 +282,7 @@ fr_status accumulate_impl(const fr_routing* R, const float* rain, float* w_out, 
     if (mfd && (area_out || !w_out)) return FR_ERR_INVALID_ARG;
     const int64_t n = R->nx * R->ny;
     if (!(mfd ? ws_ok_mfd(ws, ws_bytes, n) : ws_ok(ws, ws_bytes, n))) return FR_ERR_WORKSPACE;
-    Prob P = base_prob(R, (char*)ws);
+    Prob P = base_prob(R, (char*)ws, w_out != nullptr);
     P.init = rain;
     P.out_hi = w_out;
     if (w_lo_out) {

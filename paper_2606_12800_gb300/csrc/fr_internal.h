@@ -44,7 +44,7 @@ struct Prob {
     // the local phase leaves at least skel_min global cells, the cell walkers
     // otherwise (~0: walkers always)
     unsigned long long skel_min;
-    uint16_t* skpool;               // dependency slots, kSkelPool per skeleton tile
+    uint16_t* skpool;               // dependency slots, skel_pool per skeleton tile
     unsigned long long* skstarts;   // exits that start a skeleton walker
     uint32_t* sktiles;              // skeleton tiles holding global cells
 };
@@ -83,13 +83,13 @@ cudaError_t read_clear_tma_error(unsigned* out, cudaStream_t s);
 // Linear receiver index of every cell from D8 codes (fr_receivers.cu).
 cudaError_t launch_receiver_index(const uint8_t* dir, int64_t nx, int64_t ny, bool wide, void* out,
                                   cudaStream_t s);
-// Skeleton tiles of the D8 global phase (fr_skel.cu): kSkelTile x kSkelTile
-// cells; kSkelPool dependency slots per tile (a dependency is a donor in the
-// one-cell ring around the tile, and each ring cell has one receiver).
-constexpr int kSkelTile = 64;
-constexpr int kSkelPool = 4 * kSkelTile + 4;
-__host__ __device__ inline int64_t skel_tiles(int64_t nx, int64_t ny) {
-    return ((nx + kSkelTile - 1) / kSkelTile) * ((ny + kSkelTile - 1) / kSkelTile);
+// Skeleton tiles of the D8 global phase (fr_skel.cu): side x side cells, with
+// water or areas alone; dependency slots per tile (a dependency is a donor in
+// the one-cell ring around the tile, and each ring cell has one receiver).
+__host__ __device__ constexpr int skel_side(bool with_water) { return with_water ? 32 : 64; }
+__host__ __device__ constexpr int skel_pool(int side) { return 4 * side + 4; }
+__host__ __device__ inline int64_t skel_tiles(int64_t nx, int64_t ny, int side) {
+    return ((nx + side - 1) / side) * ((ny + side - 1) / side);
 }
 // Skeleton solve of the global cells left by the D8 forward local phase;
 // every kernel returns at once unless the global-cell count reaches

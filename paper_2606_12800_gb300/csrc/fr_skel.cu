@@ -9,7 +9,7 @@
 // cells are the river trunks, thousands of cells long, and a walker that
 // follows a trunk one cell per dependent step takes tens to hundreds of
 // milliseconds.  This file solves the same global cells exactly on the
-// skeleton of a second, non-overlapping decomposition into 64x64 tiles, the
+// skeleton of a second, non-overlapping decomposition into tiles (SkGeo), the
 // solve on "the skeleton of the domain decomposition" that Sec. 2.4 mentions,
 // made exact for single-receiver routing:
 //
@@ -50,11 +50,22 @@
 namespace fr {
 namespace {
 
-constexpr int SX = kSkelTile, SY = kSkelTile, SN = SX * SY;
-constexpr int SRX = SX + 2, SRY = SY + 2, SRN = SRX * SRY;  // with a one-cell ring
-constexpr int kSkNT = 256;
-static_assert(SN <= 4096, "local indices take 12 bits");
-static_assert(kSkelPool == 2 * (SX + SY) + 4, "dependency slots per tile: the ring cells");
+// Tile sides.  Areas alone: 64 (three blocks of 256 threads per SM; 32 measured
+// the same in the tile passes, with twice the steps in between).  With water a
+// cell takes 28 bytes of shared memory, so a 64x64 tile leaves room for one
+// block per SM and its chain of latencies is exposed: 32x32 tiles, six blocks of
+// 128 threads, took passes A and C of a filled 4096^2 DEM from 922 and 773 to
+// 331 and 289 us.
+template <bool W>
+struct SkGeo {
+    static constexpr int SX = skel_side(W), SY = SX, SN = SX * SY;
+    static constexpr int SRX = SX + 2, SRY = SY + 2, SRN = SRX * SRY;  // with a one-cell ring
+    static constexpr int NT = W ? 128 : 256;                           // threads of the tile passes
+    static constexpr int kBlocks = W ? 6 : 3;                          // blocks per SM asked of the compiler
+    static constexpr int kPool = skel_pool(SX);
+    static_assert(SN <= 4096, "local indices take 12 bits");
+    static_assert(kPool == 2 * (SX + SY) + 4, "dependency slots per tile: the ring cells");
+};
 
 // Cell byte of the ring arrays: the receiver code (bits 0-3; 15 = none, also
 // for receivers outside the grid) and the global flag.
@@ -77,11 +88,14 @@ constexpr uint16_t kPtrFinal = 1u << 12, kPtrExit = 1u << 13;
 
 // Link word of a boundary cell (per cell, 8 bytes, in the workspace):
 //   exit:   kind 2, pending dependencies (bits 0-15), list begin (16-31),
-//           list length (32-47);
+//           list length (32-47) (areas alone: see kLkSum);
 //   entry:  kind 1, the exit its in-tile path reaches (cell index, bits 0-39);
 //   else 0 (an entry whose path ends inside its tile).
 constexpr unsigned long long kLkExit = 2ull << 62, kLkEntry = 1ull << 62, kLkKind = 3ull << 62;
 constexpr unsigned long long kLkCell = (1ull << 40) - 1;
+// Areas alone: an exit's word holds its sum (bits 0-47) and its pending
+// dependencies (48-59) instead.
+constexpr unsigned long long kLkSum = (1ull << 48) - 1, kLkOne = 1ull << 48, kLkPend = 0xFFFull << 48;
 // Pending count of an exit whose in-tile partial value was never computed (a
 // cycle upstream of it inside its tile): never reached by arrivals.
 constexpr unsigned long long kLkNever = 0xFFFFull;
@@ -92,7 +106,9 @@ struct TileGeo {
     int tiles_x;
 };
 
+template <bool W>
 __device__ __forceinline__ TileGeo tile_geo(const Prob& P, int64_t t) {
+    constexpr int SX = SkGeo<W>::SX, SY = SkGeo<W>::SY;
     TileGeo g;
     g.tiles_x = (int)((P.nx + SX - 1) / SX);
     const int64_t ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
@@ -132,7 +148,9 @@ __device__ __forceinline__ int bindex(int lx, int ly, int ex, int ey) {
 }
 
 template <bool W, bool AREA>
-struct SmemSk {
+struct SmemSk : SkGeo<W> {
+    using Geo = SkGeo<W>;
+    static constexpr int SX = Geo::SX, SN = Geo::SN, SRN = Geo::SRN, kSkNT = Geo::NT;
     static constexpr bool kPush = AREA && !W;
     uint8_t cg[SRN];                                    // ring layout: code | kGlob
     uint8_t dm[kPush ? 1 : SN];                         // pull: in-tile global donors (codes)
@@ -167,6 +185,8 @@ __device__ __forceinline__ bool in_ext(int lx, int ly, const TileGeo& g) {
 // row-major order (S.gl, S.ng).
 template <class S_>
 __device__ void load_tile(S_& S, const Prob& P, const TileGeo& g) {
+    constexpr int SX = S_::SX, SY = S_::SY, SN = S_::SN, SRX = S_::SRX, SRY = S_::SRY, SRN = S_::SRN;
+    constexpr int kSkNT = S_::kSkNT;
     // interior tiles of a grid whose rows are 32-cell aligned: 16-byte code
     // chunks and one word of global bits per chunk (grid x in [x0 - 16, x0 + 80))
     if (g.ex == SX && g.ey == SY && (P.nx & 31) == 0 && ((uintptr_t)P.rb & 15) == 0 && g.x0 >= 16 &&
@@ -324,7 +344,9 @@ __device__ __forceinline__ void hand_out_filtered(S_& S, int ng, int& c, bool& m
 // Successor word of global cell c (local index; ring index r): its in-tile
 // global receiver, or c itself marked final (and exit if the receiver is a
 // global cell of another tile).
+template <class S_>
 __device__ __forceinline__ uint16_t succ_word(const uint8_t* cg, int c, int r, const TileGeo& g) {
+    constexpr int SX = S_::SX, SRX = S_::SRX;
     const int ly = c / SX, lx = c - ly * SX;
     const int k = cg[r] & 15;
     if (k < 8 && (cg[r + offy(k) * SRX + offx(k)] & kGlob)) {
@@ -403,6 +425,7 @@ __device__ __forceinline__ int cw_j(unsigned long long w) { return (int)((w >> 4
 
 template <class S_>
 __device__ void contract_push(S_& S, int ng) {
+    constexpr int kSkNT = S_::kSkNT;
     const int tid = threadIdx.x;
     // 1. chain cells take their donor
     for (int i = tid; i < ng; i += kSkNT) {
@@ -520,6 +543,7 @@ __device__ void contract_push(S_& S, int ng) {
 // written before its arrival, the completing thread reads them after).
 template <bool AREA, class S_>
 __device__ void walk_pull(S_& S) {
+    constexpr int SX = S_::SX;
     const int nst = S.qtail;
     int c = -1;
     bool more = true;
@@ -563,12 +587,13 @@ __device__ void walk_pull(S_& S) {
 
 // Tiles holding at least one global cell, listed once per call (one warp per
 // tile reads the tile's rows of the global-cell bits).
+template <bool W>
 __global__ void __launch_bounds__(256) k_skel_tiles(Prob P, EngineGlobals* G, int64_t ntiles) {
     if (__ldcg(&G->glist_count) < P.skel_min) return;
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x / 32);
     for (int64_t t = (int64_t)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); t < ntiles; t += warps) {
-        const TileGeo g = tile_geo(P, t);
+        const TileGeo g = tile_geo<W>(P, t);
         uint32_t any = 0;
         for (int ly = lane; ly < g.ey; ly += 32) {
             const int64_t b0 = (g.y0 + ly) * P.nx + g.x0, b1 = b0 + g.ex;  // bits [b0, b1)
@@ -589,8 +614,9 @@ __global__ void __launch_bounds__(256) k_skel_tiles(Prob P, EngineGlobals* G, in
 
 // Pass A: in-tile partial values, exits, entries and dependency lists.
 template <bool W, bool AREA>
-__global__ void __launch_bounds__(kSkNT, 3) k_skel_a(Prob P, EngineGlobals* G) {
+__global__ void __launch_bounds__(SkGeo<W>::NT, SkGeo<W>::kBlocks) k_skel_a(Prob P, EngineGlobals* G) {
     using Sm = SmemSk<W, AREA>;
+    constexpr int SX = Sm::SX, SRX = Sm::SRX, kSkNT = Sm::kSkNT, kSkelPool = Sm::kPool;
     constexpr bool kPush = Sm::kPush;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Sm& S = *reinterpret_cast<Sm*>(smem_raw);
@@ -599,7 +625,7 @@ __global__ void __launch_bounds__(kSkNT, 3) k_skel_a(Prob P, EngineGlobals* G) {
     const int tid = threadIdx.x;
     for (unsigned long long it = blockIdx.x; it < ntl; it += gridDim.x) {
         const int64_t t = (int64_t)__ldcg(P.sktiles + it);
-        const TileGeo g = tile_geo(P, t);
+        const TileGeo g = tile_geo<W>(P, t);
         __syncthreads();  // the previous tile's shared memory is no longer read
         if (tid == 0) {
             S.qtail = 0;
@@ -656,7 +682,7 @@ __global__ void __launch_bounds__(kSkNT, 3) k_skel_a(Prob P, EngineGlobals* G) {
                 }
                 const uint32_t nin = __popc(din);
                 S.nin[c] = (uint8_t)nin;
-                S.sc[c] = succ_word(S.cg, c, r, g);
+                S.sc[c] = succ_word<Sm>(S.cg, c, r, g);
                 if constexpr (kPush) {
                     S.pw[c] = (unsigned long long)(kDone - nin) << 56 | a;
                 } else {
@@ -781,13 +807,17 @@ __global__ void __launch_bounds__(kSkNT, 3) k_skel_a(Prob P, EngineGlobals* G) {
             const bool exit = (p & kPtrExit) && (p & 0xFFF) == c;
             const int nd = S.bnd[b];
             if (exit) {
+                if (FR_OK(gi, ncell(P), 41)) reinterpret_cast<uint8_t*>(P.cnt)[gi] = 0;  // not done yet (pass B)
                 const unsigned long long len = kPush ? (unsigned long long)S.bdep[b] : S.bslots[b];
                 bool fin;
                 if constexpr (kPush) fin = (S.pw[c] >> 56) == kDone;
                 else fin = (S.pk[c] & kFin) != 0;
-                const unsigned long long pend = fin ? len : kLkNever;
-                const unsigned long long beg = kPush ? 0ull : S.bbeg[b];
-                P.link[gi] = (int64_t)(kLkExit | pend | (beg << 16) | (len << 32));
+                if constexpr (kPush) {
+                    P.link[gi] = (int64_t)(kLkExit | (fin ? len * kLkOne : kLkPend) | (S.pw[c] & kPwVal));
+                } else {
+                    const unsigned long long pend = fin ? len : kLkNever;
+                    P.link[gi] = (int64_t)(kLkExit | pend | ((unsigned long long)S.bbeg[b] << 16) | (len << 32));
+                }
                 if (fin && len == 0) {
                     const unsigned long long slot = atomicAdd(&G->fcount[0], 1ull);
                     P.skstarts[slot] = (unsigned long long)gi;
@@ -831,61 +861,111 @@ __global__ void __launch_bounds__(kSkNT, 3) k_skel_a(Prob P, EngineGlobals* G) {
     }
 }
 
-// Pass B: walkers over the exits.
+// The exit that water leaving exit x by code k reaches (an exit of the next
+// tile, itself or through an entry), or -1.  The words read are constant after
+// pass A but for an exit's counts.
+__device__ __forceinline__ int64_t next_exit(const Prob& P, int64_t x, uint32_t k) {
+    if (k >= 8) return -1;
+    const int64_t s = x + offi((int)k, P.nx);
+    const unsigned long long rs = __ldcg(reinterpret_cast<const unsigned long long*>(P.link) + s);
+    const int64_t q = (rs & kLkKind) == kLkExit ? s : (rs & kLkKind) == kLkEntry ? (int64_t)(rs & kLkCell) : -1;
+    return q >= 0 && FR_OK(q, ncell(P), 42) ? q : -1;
+}
+
+// Pass B: walkers over the exits.  A river that crosses T tiles takes T
+// dependent steps, so a step's latency is what counts.  Areas alone: an exit's
+// word holds its pending count and its sum, and one atomic does an arrival
+// (two trips to L2 per step; areas and counts apart, with the ordering between
+// them, took four).  With water the dependencies are pulled in list order,
+// their slots and values loaded eight at a time.
+// Filled 8192^2, areas 514 -> 351 us; filled 4096^2, water and areas in 32x32 tiles
+// 956 -> 624 us.
 template <bool W, bool AREA>
 __global__ void __launch_bounds__(256) k_skel_walk(Prob P, EngineGlobals* G) {
     if (__ldcg(&G->glist_count) < P.skel_min) return;
+    using Geo = SkGeo<W>;
+    constexpr int SX = Geo::SX, SY = Geo::SY, SRX = Geo::SRX;
     const unsigned long long count = __ldcg(&G->fcount[0]);
     const int tiles_x = (int)((P.nx + SX - 1) / SX);
     uint8_t* done = reinterpret_cast<uint8_t*>(P.cnt);
+    unsigned long long* link = reinterpret_cast<unsigned long long*>(P.link);
     for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += (unsigned long long)gridDim.x * blockDim.x) {
         int64_t x = (int64_t)__ldcg(P.skstarts + i);
         if constexpr (AREA && !W) {
-            // areas alone: every dependency adds its total into the exit's
-            // area (exact integer atomics, any order), so the arrival that
-            // completes the count finds the exit's total there
+            uint32_t k = rd_rb(P, x);
+            unsigned long long a = __ldcg(link + x) & kLkSum;
             for (;;) {
-                const uint8_t k = rd_rb(P, x);
-                const unsigned long long a = rd_area(P, x);
+                wr_area(P, x, a);
                 if (FR_OK(x, ncell(P), 41)) done[x] = 1;
-                if (k >= 8) break;
-                const int64_t s = x + offi(k, P.nx);
-                const unsigned long long rs = (unsigned long long)__ldcg(
-                    reinterpret_cast<const unsigned long long*>(P.link) + s);
-                int64_t q;
-                if ((rs & kLkKind) == kLkExit) q = s;
-                else if ((rs & kLkKind) == kLkEntry) q = (int64_t)(rs & kLkCell);
-                else break;
-                if (!FR_OK(q, ncell(P), 42)) break;
-                atomicAdd(reinterpret_cast<unsigned long long*>(P.area) + q, a);
-                cuda::atomic_ref<unsigned long long, cuda::thread_scope_device> at(
-                    reinterpret_cast<unsigned long long*>(P.link)[q]);
-                const unsigned long long old = at.fetch_sub(1ull, cuda::memory_order_acq_rel);
-                if ((old & 0xFFFFull) != 1ull) break;
+                const int64_t q = next_exit(P, x, k);
+                if (q < 0) break;
+                const uint32_t kq = rd_rb(P, q);
+                const unsigned long long old = atomicAdd(link + q, a - kLkOne);
+                if ((old & kLkPend) != kLkOne) break;
+                a = (old + a) & kLkSum;
                 x = q;
+                k = kq;
             }
         } else {
-            for (;;) {
-                const uint8_t k = rd_rb(P, x);
-                const unsigned long long rec = (unsigned long long)__ldcg(
-                    reinterpret_cast<const unsigned long long*>(P.link) + x);
+            // what exit x's step reads and no other exit changes: its partial
+            // value, its word, the dependencies' slots (the first eight)
+            struct Exit {
+                unsigned long long rec, a;
+                df v;
+                uint32_t k;
+                int j[8];
+            };
+            auto load1 = [&](int64_t y, Exit& e) {
+                e.rec = __ldcg(link + y);
+                e.k = rd_rb(P, y);
+                e.v = W ? df{rd_cg(P.out_hi, P, y, 35), rd_cg(P.out_lo, P, y, 36)} : df_make(0.0f);
+                e.a = AREA ? rd_area(P, y) : 0ull;
+            };
+            auto slots = [&](int64_t y, unsigned long long rec, int s0, int64_t& origin, int (&j)[8]) {
                 const int begin = (int)((rec >> 16) & 0xFFFF), len = (int)((rec >> 32) & 0xFFFF);
-                const int64_t yy = x / P.nx, xx = x - yy * P.nx;
-                const int64_t tx = xx / SX, ty = yy / SY;
-                const int64_t ox = tx * SX - 1, oy = ty * SY - 1;  // ring origin of x's tile
-                const uint16_t* pool = P.skpool + (ty * tiles_x + tx) * kSkelPool;
-                df v = df_make(0.0f);
-                unsigned long long a = 0;
-                if constexpr (W) v = df{rd_cg(P.out_hi, P, x, 35), rd_cg(P.out_lo, P, x, 36)};
-                if constexpr (AREA) a = rd_area(P, x);
-    #pragma unroll 1
-                for (int s = 0; s < len; ++s) {
-                    const int j = __ldcg(pool + begin + s);
-                    const int ry = j / SRX, rx = j - ry * SRX;
-                    const int64_t y = (oy + ry) * P.nx + (ox + rx);
-                    if constexpr (W) v = df_add(v, df{rd_cg(P.out_hi, P, y, 37), rd_cg(P.out_lo, P, y, 38)});
-                    if constexpr (AREA) a += rd_area(P, y);
+                const int64_t yy = y / P.nx, xx = y - yy * P.nx, tx = xx / SX, ty = yy / SY;
+                origin = (ty * SY - 1) * P.nx + tx * SX - 1;  // ring origin of y's tile
+                const uint16_t* pool = P.skpool + (ty * tiles_x + tx) * Geo::kPool + begin + s0;
+#pragma unroll
+                for (int s = 0; s < 8; ++s) j[s] = s0 + s < len ? (int)__ldcg(pool + s) : -1;
+                return len;
+            };
+            Exit e;
+            load1(x, e);
+            int64_t origin, q = next_exit(P, x, e.k);
+            int len = slots(x, e.rec, 0, origin, e.j);
+            for (;;) {
+                df v = e.v;
+                unsigned long long a = e.a;
+                Exit n;
+                for (int s0 = 0;;) {
+                    float h[8], l[8];
+                    unsigned long long b[8];
+#pragma unroll
+                    for (int s = 0; s < 8; ++s) {
+                        h[s] = l[s] = 0.0f;
+                        b[s] = 0;
+                        if (e.j[s] < 0) continue;
+                        const int ry = e.j[s] / SRX, rx = e.j[s] - ry * SRX;
+                        const int64_t y = origin + ry * P.nx + rx;
+                        if constexpr (W) {
+                            h[s] = rd_cg(P.out_hi, P, y, 37);
+                            l[s] = rd_cg(P.out_lo, P, y, 38);
+                        }
+                        if constexpr (AREA) b[s] = rd_area(P, y);
+                    }
+                    // the next exit's own loads travel with these
+                    if (s0 == 0 && q >= 0) load1(q, n);
+#pragma unroll
+                    for (int s = 0; s < 8; ++s) {
+                        if (e.j[s] < 0) continue;
+                        if constexpr (W) v = df_add(v, df{h[s], l[s]});
+                        a += b[s];
+                    }
+                    s0 += 8;
+                    if (s0 >= len) break;
+                    slots(x, e.rec, s0, origin, e.j);
                 }
                 if constexpr (W) {
                     wr_f(P.out_hi, P, x, v.hi, 39);
@@ -893,22 +973,17 @@ __global__ void __launch_bounds__(256) k_skel_walk(Prob P, EngineGlobals* G) {
                 }
                 if constexpr (AREA) wr_area(P, x, a);
                 if (FR_OK(x, ncell(P), 41)) done[x] = 1;
-                // the exit reached from this exit's receiver (an entry of the next tile)
-                if (k >= 8) break;
-                const int64_t s = x + offi(k, P.nx);
-                const unsigned long long rs = (unsigned long long)__ldcg(
-                    reinterpret_cast<const unsigned long long*>(P.link) + s);
-                int64_t q;
-                if ((rs & kLkKind) == kLkExit) q = s;
-                else if ((rs & kLkKind) == kLkEntry) q = (int64_t)(rs & kLkCell);
-                else break;
-                if (!FR_OK(q, ncell(P), 42)) break;
+                if (q < 0) break;
+                // beside the ordering and the arrival: the next exit's slots
+                const int64_t q2 = next_exit(P, q, n.k);
+                len = slots(q, n.rec, 0, origin, n.j);
                 // release this exit's value; the completing arrival acquires all
-                cuda::atomic_ref<unsigned long long, cuda::thread_scope_device> at(
-                    reinterpret_cast<unsigned long long*>(P.link)[q]);
+                cuda::atomic_ref<unsigned long long, cuda::thread_scope_device> at(link[q]);
                 const unsigned long long old = at.fetch_sub(1ull, cuda::memory_order_acq_rel);
                 if ((old & 0xFFFFull) != 1ull) break;
                 x = q;
+                q = q2;
+                e = n;
             }
         }
     }
@@ -917,9 +992,10 @@ __global__ void __launch_bounds__(256) k_skel_walk(Prob P, EngineGlobals* G) {
 // Pass C: inflows of the entries passed down the in-tile receivers; final
 // values of the global cells; completion count.
 template <bool W, bool AREA>
-__global__ void __launch_bounds__(kSkNT, 3) k_skel_fix(Prob P, EngineGlobals* G,
+__global__ void __launch_bounds__(SkGeo<W>::NT, SkGeo<W>::kBlocks) k_skel_fix(Prob P, EngineGlobals* G,
                                                    unsigned long long total_cells) {
     using Sm = SmemSk<W, AREA>;
+    constexpr int SX = Sm::SX, SRX = Sm::SRX, kSkNT = Sm::kSkNT;
     constexpr bool kPush = Sm::kPush;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Sm& S = *reinterpret_cast<Sm*>(smem_raw);
@@ -930,7 +1006,7 @@ __global__ void __launch_bounds__(kSkNT, 3) k_skel_fix(Prob P, EngineGlobals* G,
     unsigned long long done = 0;
     for (unsigned long long it = blockIdx.x; it < ntl; it += gridDim.x) {
         const int64_t t = (int64_t)__ldcg(P.sktiles + it);
-        const TileGeo g = tile_geo(P, t);
+        const TileGeo g = tile_geo<W>(P, t);
         __syncthreads();
         if (tid == 0) {
             S.qtail = 0;
@@ -1016,7 +1092,7 @@ __global__ void __launch_bounds__(kSkNT, 3) k_skel_fix(Prob P, EngineGlobals* G,
                 }
                 const uint32_t nin = __popc(din);
                 S.nin[c] = (uint8_t)nin;
-                S.sc[c] = succ_word(S.cg, c, r, g);
+                S.sc[c] = succ_word<Sm>(S.cg, c, r, g);
                 if constexpr (kPush) {
                     S.pw[c] = (unsigned long long)(kDone - nin) << 56 | ((fl & kPoison) ? kPwPois : 0ull) | a;
                 } else {
@@ -1121,11 +1197,11 @@ __global__ void __launch_bounds__(kSkNT, 3) k_skel_fix(Prob P, EngineGlobals* G,
 }
 
 template <class K>
-int persistent_grid(K kernel, size_t smem) {
+int persistent_grid(K kernel, int threads, size_t smem) {
     int dev = 0, sms = 0, per = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, kSkNT, smem) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem) != cudaSuccess) return 0;
     return sms * (per > 0 ? per : 1);
 }
 
@@ -1138,20 +1214,21 @@ cudaError_t launch_skel_t(const Prob& P, EngineGlobals* G, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     e = smem_limit_once(k_skel_fix<W, AREA>, sm, set_c);
     if (e != cudaSuccess) return e;
-    if (!grid_a) grid_a = persistent_grid(k_skel_a<W, AREA>, sm);
-    if (!grid_c) grid_c = persistent_grid(k_skel_fix<W, AREA>, sm);
+    if (!grid_a) grid_a = persistent_grid(k_skel_a<W, AREA>, SkGeo<W>::NT, sm);
+    if (!grid_c) grid_c = persistent_grid(k_skel_fix<W, AREA>, SkGeo<W>::NT, sm);
     if (!grid_a || !grid_c) return cudaErrorInvalidConfiguration;
-    const int64_t ntiles = skel_tiles(P.nx, P.ny);
+    const int64_t ntiles = skel_tiles(P.nx, P.ny, skel_side(W));
+    constexpr int kSkNT = SkGeo<W>::NT;
     int tgrid = (int)((ntiles + 7) / 8);
     if (tgrid > 16 * 152) tgrid = 16 * 152;
     if (tgrid < 1) tgrid = 1;
-    k_skel_tiles<<<tgrid, 256, 0, s>>>(P, G, ntiles);
+    k_skel_tiles<W><<<tgrid, 256, 0, s>>>(P, G, ntiles);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_skel_a<W, AREA><<<grid_a, kSkNT, sm, s>>>(P, G);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_skel_walk<W, AREA><<<walker_grid(), 256, 0, s>>>(P, G);
+    k_skel_walk<W, AREA><<<walker_grid() / 2, 256, 0, s>>>(P, G);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_skel_fix<W, AREA><<<grid_c, kSkNT, sm, s>>>(P, G, (unsigned long long)(P.nx * P.ny));
