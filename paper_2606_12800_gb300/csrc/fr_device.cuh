@@ -117,23 +117,36 @@ __device__ __forceinline__ uint8_t d8_code(float zc, const float (&zn)[8], float
     return code;
 }
 
-// The same selection without branches, for the rule fixed at compile time:
-// d = fl32(zc - zk) > 0 exactly when zk < zc (a difference of two floats is
-// zero only if they are equal; infinities and NaN compare false as above).
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));  // of NaN and a number, the number
+    return r;
+}
+
+// The same selection for the rule fixed at compile time: the largest of the
+// eight keys s_k by three-input maxima, then the first code that has it (a NaN
+// key equals nothing).  A positive largest key belongs to a lower neighbour and
+// a negative one to none; a zero or NaN one (returned in m) leaves the choice to
+// d8_code: the neighbours are level, or a drop has underflowed.
 template <bool LOWEST>
-__device__ __forceinline__ uint32_t d8_code_sel(float zc, const float (&zn)[8], float c_orth,
-                                                float c_diag) {
-    float best = -1.0f;
-    uint32_t code = kSink;
+__device__ __forceinline__ uint32_t d8_code_max(float zc, const float (&zn)[8], float c_orth,
+                                                float c_diag, float& m) {
+    float s[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
         const float d = __fsub_rn(zc, zn[k]);
-        const float s = LOWEST ? d : __fmul_rn(d, k < 4 ? c_orth : c_diag);
-        const bool take = (d > 0.0f) & (s > best);
-        best = take ? s : best;
-        code = take ? (uint32_t)k : code;
+        s[k] = LOWEST ? d : __fmul_rn(d, k < 4 ? c_orth : c_diag);
     }
-    return code;
+    m = max3(max3(s[0], s[1], s[2]), max3(s[3], s[4], s[5]), fmaxf(s[6], s[7]));
+    uint32_t code = 7;
+#pragma unroll
+    for (int k = 6; k >= 0; --k) code = s[k] == m ? (uint32_t)k : code;
+    return m > 0.0f ? code : kSink;
+}
+// Whether one of four largest keys is zero or NaN (or so small that their
+// product underflows): their cells are chosen again by d8_code.
+__device__ __forceinline__ bool d8_unsure(const float (&m)[4]) {
+    return !(fabsf(__fmul_rn(__fmul_rn(m[0], m[1]), __fmul_rn(m[2], m[3]))) > 0.0f);
 }
 
 // ------------------------------------------------------------ MFD weights

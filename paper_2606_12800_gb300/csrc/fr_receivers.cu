@@ -1,11 +1,13 @@
 // fr_receivers.cu -- local flow routing kernels (paper Sec. 2.1 for D8,
 // App. A for the multi-receiver split).
 //
-// Each CTA stages a (TY+4) x (TX+4) elevation tile (two-cell halo) in shared
-// memory, computes the routing byte of the tile plus a one-cell ring, and from
-// the ring the number of donors of each tile cell.  Outside the grid the tile
-// holds +inf, which is never strictly lower than anything.
+// Codes alone come from the TMA-pipelined kernel, or by warps marching down
+// strips where TMA cannot address the grid; donor counts, D-infinity and batched
+// slope splits from blocks that stage a (TY+4) x (TX+4) elevation tile (two-cell
+// halo) in shared memory, which outside the grid holds +inf, never strictly lower
+// than anything.
 #include <cmath>
+#include <type_traits>
 
 #include "fr_internal.h"
 #include "fr_tma.cuh"
@@ -47,10 +49,115 @@ __device__ __forceinline__ void tile_origin(int64_t nx, int64_t& x0, int64_t& y0
     y0 = ty * RTY;
 }
 
-// D8 codes of RTX x RTY tile cells; each thread computes four consecutive
-// cells of a row from a 3 x 6 register window.  Tiles away from the grid
-// boundary skip all edge and bounds tests.
-template <bool INDEG, bool LOWEST>
+constexpr int kStrip = 4;  // rows of a strip (a tile is RTY / kStrip strips)
+
+// D8 codes of RTX x kStrip cells by one warp, without shared memory or
+// barriers: lane l holds columns l, l + 32, l + 64 and l + 96 and marches down
+// the rows with three rows in registers, neighbours along a row coming by
+// shuffles.  For grids TMA cannot address and for batches: every load is
+// coalesced whatever the rows' alignment.  Bound by instruction issue.  1537x2603
+// 23 us by staged tiles, 19 us; batch of 32 tiles, 18 M cells, 160 us by staged
+// tiles of a block, 83 us (strips of 16 rows loaded as they go 116 us).
+template <bool LOWEST, bool D4, bool INTERIOR>
+__device__ __forceinline__ void recv_d8_strip_t(const float* __restrict__ z, int64_t nx, int64_t ny,
+                                              float c_orth, float c_diag, bool edge_route,
+                                              uint8_t* __restrict__ dir, int64_t x0, int64_t y0) {
+    static_assert(RTX == 128, "four columns a lane");
+    const float inf = __int_as_float(0x7f800000);
+    const int lane = threadIdx.x & 31;
+    struct Row {
+        float v[4], e;  // the lane's cells; lanes 0 and 31: the cell beside the strip
+    };
+    auto load = [&](int64_t gy, Row& w) {
+        const bool row = INTERIOR || (gy >= 0 && gy < ny);
+        const float* p = z + gy * nx + x0 + lane;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) w.v[g] = INTERIOR || (row && x0 + lane + 32 * g < nx) ? __ldg(p + 32 * g) : inf;
+        w.e = inf;
+        if ((lane == 0 || lane == 31) && row && (INTERIOR || (lane ? x0 + RTX < nx : x0 > 0)))
+            w.e = __ldg(p + (lane ? 97 : -1));
+    };
+    struct Win {
+        float l[4], c[4], r[4];
+    };
+    auto spread = [&](const Row& w, Win& n) {
+        float up[4], dn[4];
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            up[g] = __shfl_sync(0xffffffffu, w.v[g], (lane + 31) & 31);
+            dn[g] = __shfl_sync(0xffffffffu, w.v[g], (lane + 1) & 31);
+            n.c[g] = w.v[g];
+        }
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            n.l[g] = lane ? up[g] : g ? up[g > 0 ? g - 1 : 0] : w.e;
+            n.r[g] = lane < 31 ? dn[g] : g < 3 ? dn[g < 3 ? g + 1 : 3] : w.e;
+        }
+    };
+    Row rows[kStrip + 2];  // all loads issued before the first is used
+#pragma unroll
+    for (int r = 0; r < kStrip + 2; ++r) load(y0 + r - 1, rows[r]);
+    Win a, b, c;
+    spread(rows[0], a);
+    spread(rows[1], b);
+#pragma unroll
+    for (int r = 0; r < kStrip; ++r) {
+        const int64_t gy = y0 + r;
+        if (!INTERIOR && gy >= ny) break;
+        spread(rows[r + 2], c);
+        uint32_t codes[4];
+        float m[4];
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            const float zn[8] = {b.r[g], a.c[g], b.l[g], c.c[g], D4 ? inf : a.r[g], D4 ? inf : a.l[g],
+                                 D4 ? inf : c.l[g], D4 ? inf : c.r[g]};
+            codes[g] = d8_code_max<LOWEST>(b.c[g], zn, c_orth, c_diag, m[g]);
+        }
+        if (d8_unsure(m)) {
+#pragma unroll 1
+            for (int g = 0; g < 4; ++g) {
+                const int64_t gx = x0 + lane + 32 * g;
+                if (gx >= nx) break;
+                float zn[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const int64_t xn = gx + offx(k), yn = gy + offy(k);
+                    zn[k] = (k >= 4 && D4) || xn < 0 || yn < 0 || xn >= nx || yn >= ny ? inf : __ldg(z + yn * nx + xn);
+                }
+                const uint32_t code = d8_code(__ldg(z + gy * nx + gx), zn, c_orth, c_diag, LOWEST);
+                codes[0] = g == 0 ? code : codes[0];
+                codes[1] = g == 1 ? code : codes[1];
+                codes[2] = g == 2 ? code : codes[2];
+                codes[3] = g == 3 ? code : codes[3];
+            }
+        }
+        uint8_t* o = dir + gy * nx + x0 + lane;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            const int64_t gx = x0 + lane + 32 * g;
+            if (!INTERIOR) {
+                if (gx >= nx) continue;
+                if (!edge_route && is_edge(gx, gy, nx, ny)) codes[g] = kSink;
+            }
+            o[32 * g] = (uint8_t)codes[g];
+        }
+        a = b;
+        b = c;
+    }
+}
+
+template <bool LOWEST, bool D4>
+__device__ __forceinline__ void recv_d8_strip(const float* __restrict__ z, int64_t nx, int64_t ny,
+                                              float c_orth, float c_diag, bool edge_route,
+                                              uint8_t* __restrict__ dir, int64_t x0, int64_t y0) {
+    if (x0 >= 1 && y0 >= 1 && x0 + RTX + 1 <= nx && y0 + kStrip + 1 <= ny)
+        recv_d8_strip_t<LOWEST, D4, true>(z, nx, ny, c_orth, c_diag, edge_route, dir, x0, y0);
+    else
+        recv_d8_strip_t<LOWEST, D4, false>(z, nx, ny, c_orth, c_diag, edge_route, dir, x0, y0);
+}
+
+// D8 codes and donor counts of RTX x RTY tile cells by a block.
+template <bool LOWEST>
 __device__ __forceinline__ void recv_d8_tile(const float* __restrict__ z, int64_t nx, int64_t ny,
                                              float c_orth, float c_diag, uint32_t flags,
                                              uint8_t* __restrict__ dir,
@@ -58,105 +165,60 @@ __device__ __forceinline__ void recv_d8_tile(const float* __restrict__ z, int64_
                                              int64_t y0) {
     __shared__ float zs[HX * HY];
     __shared__ uint8_t ds[RX * RY];
-    const bool lowest = LOWEST;
     const bool edge_route = flags & kEdgeRoute;
     const bool d4 = flags & kD4;
     const float inf = __int_as_float(0x7f800000);
-    const bool interior = x0 >= 2 && y0 >= 2 && x0 + RTX + 2 <= nx && y0 + RTY + 2 <= ny;
-    if (interior) {
-        // row by row: a warp per row, lanes along it
-        const float* base = z + (y0 - 2) * nx + (x0 - 2);
-        const int lane = threadIdx.x & 31;
-        for (int ly = threadIdx.x >> 5; ly < HY; ly += RNT / 32) {
-            const float* row = base + (int64_t)ly * nx;
-#pragma unroll
-            for (int lx = lane; lx < HX; lx += 32) zs[ly * HX + lx] = __ldg(row + lx);
-        }
-    } else {
-        load_z_tile(zs, z, nx, ny, x0, y0);
-    }
+    load_z_tile(zs, z, nx, ny, x0, y0);
     __syncthreads();
-    // four cells per thread: tile row r = (t >> 5) + 8 j, columns 4 (t & 31) .. + 3
-    const int qx = (threadIdx.x & 31) * 4;
-    for (int r = threadIdx.x >> 5; r < RTY; r += RNT / 32) {
-        float w[3][6];
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 6; ++b) w[a][b] = zs[(r + 1 + a) * HX + qx + 1 + b];
-        uint32_t packed = 0;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            uint8_t code;
-            if (!d4) {  // uniform over the launch: the common path carries no selects
-                const float zn[8] = {w[1][q + 2], w[0][q + 1], w[1][q], w[2][q + 1],
-                                     w[0][q + 2], w[0][q], w[2][q], w[2][q + 2]};
-                code = (uint8_t)d8_code_sel<LOWEST>(w[1][q + 1], zn, c_orth, c_diag);
-            } else {
-                // D4: the diagonals read +inf, which is never strictly lower
-                const float zn[8] = {w[1][q + 2], w[0][q + 1], w[1][q], w[2][q + 1], inf, inf, inf, inf};
-                code = (uint8_t)d8_code_sel<LOWEST>(w[1][q + 1], zn, c_orth, c_diag);
-            }
-            if (!interior) {  // interior tiles hold no edge cell and no cell off the grid
-                const int64_t gx = x0 + qx + q, gy = y0 + r;
-                if (gx >= nx || gy >= ny || (!edge_route && is_edge(gx, gy, nx, ny))) code = kSink;
-            }
-            packed |= (uint32_t)code << (8 * q);
-            if (INDEG) ds[(r + 1) * RX + qx + q + 1] = code;
-        }
-        const int64_t gy = y0 + r;
-        if (gy < ny) {
-            const int64_t gi = gy * nx + x0 + qx;
-            if (interior && ((uintptr_t)(dir + gi) & 3) == 0) {
-                *reinterpret_cast<uint32_t*>(dir + gi) = packed;
-            } else {
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    if (x0 + qx + q < nx) dir[gi + q] = (uint8_t)(packed >> (8 * q));
-            }
-        }
-    }
-    if (INDEG) {
-        // the ring around the tile, then the donor counts
-        for (int i = threadIdx.x; i < 2 * RX + 2 * RTY; i += RNT) {
-            int ry, rx;
-            if (i < RX) { ry = 0; rx = i; }
-            else if (i < 2 * RX) { ry = RY - 1; rx = i - RX; }
-            else if (i < 2 * RX + RTY) { ry = i - 2 * RX + 1; rx = 0; }
-            else { ry = i - 2 * RX - RTY + 1; rx = RX - 1; }
-            const int64_t gx = x0 + rx - 1, gy = y0 + ry - 1;
-            uint8_t code = kSink;
-            if (gx >= 0 && gy >= 0 && gx < nx && gy < ny &&
-                (edge_route || !is_edge(gx, gy, nx, ny))) {
+    // codes of the tile and the ring around it, then the donor counts
+    for (int i = threadIdx.x; i < RX * RY; i += RNT) {
+        const int ry = i / RX, rx = i - ry * RX;
+        const int64_t gx = x0 + rx - 1, gy = y0 + ry - 1;
+        uint8_t code = kSink;
+        if (gx >= 0 && gy >= 0 && gx < nx && gy < ny) {
+            if (edge_route || !is_edge(gx, gy, nx, ny)) {
                 float zn[8];
                 gather8(zs, rx, ry, zn);
                 if (d4) zn[4] = zn[5] = zn[6] = zn[7] = inf;
-                code = d8_code(zs[(ry + 1) * HX + (rx + 1)], zn, c_orth, c_diag, lowest);
+                code = d8_code(zs[(ry + 1) * HX + (rx + 1)], zn, c_orth, c_diag, LOWEST);
             }
-            ds[ry * RX + rx] = code;
+            if (rx >= 1 && rx <= RTX && ry >= 1 && ry <= RTY) dir[gy * nx + gx] = code;
         }
-        __syncthreads();
-        for (int i = threadIdx.x; i < RTX * RTY; i += RNT) {
-            const int ly = i / RTX, lx = i - ly * RTX;
-            const int64_t gx = x0 + lx, gy = y0 + ly;
-            if (gx >= nx || gy >= ny) continue;
-            int n = 0;
+        ds[ry * RX + rx] = code;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < RTX * RTY; i += RNT) {
+        const int ly = i / RTX, lx = i - ly * RTX;
+        const int64_t gx = x0 + lx, gy = y0 + ly;
+        if (gx >= nx || gy >= ny) continue;
+        int n = 0;
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
-                n += ds[(ly + 1 + offy(k)) * RX + (lx + 1 + offx(k))] == (uint8_t)opp(k);
-            indeg[gy * nx + gx] = (uint8_t)n;
-        }
+        for (int k = 0; k < 8; ++k)
+            n += ds[(ly + 1 + offy(k)) * RX + (lx + 1 + offx(k))] == (uint8_t)opp(k);
+        indeg[gy * nx + gx] = (uint8_t)n;
     }
 }
 
-template <bool INDEG, bool LOWEST>
+template <bool LOWEST>
+__global__ void __launch_bounds__(RNT) k_receivers_d8_indeg(const float* __restrict__ z, int64_t nx,
+                                                            int64_t ny, float c_orth, float c_diag,
+                                                            uint32_t flags, uint8_t* __restrict__ dir,
+                                                            uint8_t* __restrict__ indeg) {
+    int64_t x0, y0;
+    tile_origin(nx, x0, y0);
+    recv_d8_tile<LOWEST>(z, nx, ny, c_orth, c_diag, flags, dir, indeg, x0, y0);
+}
+
+// A strip per warp.
+template <bool LOWEST, bool D4>
 __global__ void __launch_bounds__(RNT) k_receivers_d8(const float* __restrict__ z, int64_t nx,
                                                       int64_t ny, float c_orth, float c_diag,
                                                       uint32_t flags, uint8_t* __restrict__ dir,
-                                                      uint8_t* __restrict__ indeg) {
-    int64_t x0, y0;
-    tile_origin(nx, x0, y0);
-    recv_d8_tile<INDEG, LOWEST>(z, nx, ny, c_orth, c_diag, flags, dir, indeg, x0, y0);
+                                                      int64_t ntiles) {
+    const int64_t t = (int64_t)blockIdx.x * (RNT / 32) + (threadIdx.x >> 5);
+    if (t >= ntiles) return;
+    const int64_t tiles_x = (nx + RTX - 1) / RTX, ty = t / tiles_x, tx = t - ty * tiles_x;
+    recv_d8_strip<LOWEST, D4>(z, nx, ny, c_orth, c_diag, flags & kEdgeRoute, dir, tx * RTX, ty * kStrip);
 }
 
 // ---------------------------------------------------------------- TMA path
@@ -165,10 +227,13 @@ __global__ void __launch_bounds__(RNT) k_receivers_d8(const float* __restrict__ 
 // arriving by TMA into one of TNS shared-memory stages while the previous tiles
 // are computed.  The box starts 4 cells left of the tile (its x coordinate a
 // multiple of 4, as TMA requires), so it is TTX + 8 wide.  The kernel is bound
-// by the ALU pipe (the compare-and-select chain of eight directions per cell);
-// 128x64 tiles in two stages (three CTAs per SM) measured 4.7 % faster than
-// 128x32 in three (four CTAs per SM) at 32768^2: fewer halo rows and fewer
-// per-tile waits and barriers.
+// by instruction issue and the ALU pipe (the eight directions' keys and their
+// selection): 32768^2 2.38 ms with a running best over the directions (66
+// instructions per cell), 2.04 ms with d8_code_max (56), 1.99 ms with two rows per
+// step (52).  128x64 tiles in
+// two stages (three CTAs per SM) measured 4.7 % faster than 128x32 in three
+// (four CTAs per SM) at 32768^2: fewer halo rows and fewer per-tile waits and
+// barriers.
 constexpr int TTX = 128, TTY = 64, TNS = 2;
 constexpr int TBX = TTX + 8, TBY = TTY + 2;
 constexpr unsigned kTileBytes = TBX * TBY * 4;
@@ -193,7 +258,7 @@ __global__ void __launch_bounds__(256) k_receivers_d8_tma(const __grid_constant_
                                                           int tiles_x, unsigned long long limit_ns) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     TmaSmem& S = *reinterpret_cast<TmaSmem*>(smem_raw);
-    const bool edge_route = flags & kEdgeRoute;
+    const bool edge_route = flags & kEdgeRoute, aligned = ((uintptr_t)dir & 3) == 0;
     const int tid = threadIdx.x;
     if (tid == 0) {
         for (int s = 0; s < TNS; ++s) mbar_init(&S.bar[s], 1);
@@ -232,54 +297,68 @@ __global__ void __launch_bounds__(256) k_receivers_d8_tma(const __grid_constant_
         const int64_t x0 = tx * TTX, y0 = ty * TTY;
         const bool interior = x0 >= 1 && y0 >= 1 && x0 + TTX + 1 <= nx && y0 + TTY + 1 <= ny;
         const float* b = S.buf[s].v;
-        for (int r = warp; r < TTY; r += 8) {
-            // 3 x 12 window: buffer rows r .. r + 2, columns qx .. qx + 11
-            // (tile column c sits at buffer column c + 4)
-            float w[3][12];
+        // two rows per step: they share two of the window's four rows.  Row width
+        // and tile origin are multiples of four (the tensor map's condition), so
+        // a group of four cells lies in the grid or outside it.
+        uint8_t* const out = dir + y0 * nx + x0 + qx;
+        const bool cols = x0 + qx < nx;
+        for (int r = 2 * warp; r < TTY; r += 16) {
+            // buffer rows r .. r + 3, columns qx + 3 .. qx + 8 (tile column c
+            // sits at buffer column c + 4)
+            float w[4][6];
 #pragma unroll
-            for (int a = 0; a < 3; ++a)
-#pragma unroll
-                for (int v = 0; v < 3; ++v) {
-                    const float4 f = *reinterpret_cast<const float4*>(b + (r + a) * TBX + qx + 4 * v);
-                    w[a][4 * v] = f.x;
-                    w[a][4 * v + 1] = f.y;
-                    w[a][4 * v + 2] = f.z;
-                    w[a][4 * v + 3] = f.w;
-                }
-            uint32_t packed = 0;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int c = q + 4;  // window column of the cell
-                float zn[8];
-                zn[0] = w[1][c + 1];
-                zn[1] = w[0][c];
-                zn[2] = w[1][c - 1];
-                zn[3] = w[2][c];
-                if (D4) {
-                    zn[4] = zn[5] = zn[6] = zn[7] = __int_as_float(0x7f800000);
-                } else {
-                    zn[4] = w[0][c + 1];
-                    zn[5] = w[0][c - 1];
-                    zn[6] = w[2][c - 1];
-                    zn[7] = w[2][c + 1];
-                }
-                uint32_t code = d8_code_sel<LOWEST>(w[1][c], zn, c_orth, c_diag);
-                if (!interior) {
-                    const int64_t gx = x0 + qx + q, gy = y0 + r;
-                    if (gx >= nx || gy >= ny || (!edge_route && is_edge(gx, gy, nx, ny))) code = kSink;
-                }
-                packed |= code << (8 * q);
+            for (int a = 0; a < 4; ++a) {
+                const float* row = b + (r + a) * TBX + qx;
+                const float4 f = *reinterpret_cast<const float4*>(row + 4);
+                w[a][0] = row[3];
+                w[a][1] = f.x;
+                w[a][2] = f.y;
+                w[a][3] = f.z;
+                w[a][4] = f.w;
+                w[a][5] = row[8];
             }
-            const int64_t gy = y0 + r;
-            const int64_t gx = x0 + qx;
-            if (gy < ny && gx < nx) {
-                const int64_t gi = gy * nx + gx;
-                if (gx + 3 < nx && ((uintptr_t)(dir + gi) & 3) == 0) {
-                    *reinterpret_cast<uint32_t*>(dir + gi) = packed;
-                } else {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                uint32_t codes[4];
+                float m[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int c = q + 1;  // window column of the cell
+                    const float inf = __int_as_float(0x7f800000);
+                    const float zn[8] = {w[h + 1][c + 1], w[h][c], w[h + 1][c - 1], w[h + 2][c],
+                                         D4 ? inf : w[h][c + 1], D4 ? inf : w[h][c - 1],
+                                         D4 ? inf : w[h + 2][c - 1], D4 ? inf : w[h + 2][c + 1]};
+                    codes[q] = d8_code_max<LOWEST>(w[h + 1][c], zn, c_orth, c_diag, m[q]);
+                }
+                if (d8_unsure(m)) {
+#pragma unroll 1
+                    for (int q = 0; q < 4; ++q) {
+                        const float* c = b + (r + h + 1) * TBX + qx + 4 + q;
+                        float zn[8];
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)
+                            zn[k] = k >= 4 && D4 ? __int_as_float(0x7f800000) : c[offy(k) * TBX + offx(k)];
+                        const uint32_t code = d8_code(*c, zn, c_orth, c_diag, LOWEST);
+                        codes[0] = q == 0 ? code : codes[0];
+                        codes[1] = q == 1 ? code : codes[1];
+                        codes[2] = q == 2 ? code : codes[2];
+                        codes[3] = q == 3 ? code : codes[3];
+                    }
+                }
+                if (!interior) {
+                    if (!cols || y0 + r + h >= ny) continue;
 #pragma unroll
                     for (int q = 0; q < 4; ++q)
-                        if (gx + q < nx) dir[gi + q] = (uint8_t)(packed >> (8 * q));
+                        if (!edge_route && is_edge(x0 + qx + q, y0 + r + h, nx, ny)) codes[q] = kSink;
+                }
+                uint8_t* const o = out + (int64_t)(r + h) * nx;
+                if (aligned) {
+                    *reinterpret_cast<uint32_t*>(o) =
+                        __byte_perm(__byte_perm(codes[0], codes[1], 0x0040), __byte_perm(codes[2], codes[3], 0x0040),
+                                    0x5410);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) o[q] = (uint8_t)codes[q];
                 }
             }
         }
@@ -538,12 +617,44 @@ __global__ void __launch_bounds__(RNT) k_mfd_fractions(const float* __restrict__
     }
 }
 
-// Batched receivers: persistent CTAs claim receiver tiles of any problem.
-// prefix[p] is the first receiver tile of problem p (prefix[nprob] = total).
-__global__ void __launch_bounds__(RNT) k_receivers_batch(int kind, const Prob* __restrict__ probs,
-                                                         const int64_t* __restrict__ prefix,
-                                                         int nprob, uint32_t flags,
-                                                         EngineGlobals* G) {
+// Problem and receiver tile number w of a batch: prefix[p] is the first tile of
+// problem p (prefix[nprob] = total).
+__device__ __forceinline__ int batch_tile(const int64_t* __restrict__ prefix, int nprob, int64_t w,
+                                          const Prob* __restrict__ probs, int64_t& x0, int64_t& y0) {
+    int lo = 0, hi = nprob - 1;  // last p with prefix[p] <= w
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (prefix[mid] <= w) lo = mid;
+        else hi = mid - 1;
+    }
+    const int64_t lt = w - prefix[lo], tiles_x = (probs[lo].nx + RTX - 1) / RTX;
+    const int64_t ty = lt / tiles_x, tx = lt - ty * tiles_x;
+    x0 = tx * RTX;
+    y0 = ty * RTY;
+    return lo;
+}
+
+// Batched D8 receivers: persistent warps take strips of any problem.
+template <bool LOWEST, bool D4>
+__global__ void __launch_bounds__(RNT) k_receivers_batch_d8(const Prob* __restrict__ probs,
+                                                            const int64_t* __restrict__ prefix,
+                                                            int nprob, uint32_t flags) {
+    constexpr int kSub = RTY / kStrip;
+    const int64_t total = prefix[nprob] * kSub;
+    for (int64_t w = (int64_t)blockIdx.x * (RNT / 32) + (threadIdx.x >> 5); w < total;
+         w += (int64_t)gridDim.x * (RNT / 32)) {
+        int64_t x0, y0;
+        const Prob& P = probs[batch_tile(prefix, nprob, w / kSub, probs, x0, y0)];
+        y0 += w % kSub * kStrip;
+        recv_d8_strip<LOWEST, D4>(P.z, P.nx, P.ny, P.mc.co_hi, P.mc.cd_hi, flags & kEdgeRoute,
+                                  const_cast<uint8_t*>(P.rb), x0, y0);
+    }
+}
+
+// Batched MFD receivers with fractions: persistent CTAs.
+__global__ void __launch_bounds__(RNT) k_receivers_batch_mfd(const Prob* __restrict__ probs,
+                                                             const int64_t* __restrict__ prefix,
+                                                             int nprob, uint32_t flags, EngineGlobals* G) {
     __shared__ int64_t s_work;
     const int64_t total = prefix[nprob];
     while (true) {
@@ -552,25 +663,10 @@ __global__ void __launch_bounds__(RNT) k_receivers_batch(int kind, const Prob* _
         const int64_t w = s_work;
         __syncthreads();
         if (w >= total) break;
-        int lo = 0, hi = nprob - 1;  // last p with prefix[p] <= w
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (prefix[mid] <= w) lo = mid;
-            else hi = mid - 1;
-        }
-        const Prob& P = probs[lo];
-        const int64_t lt = w - prefix[lo];
-        const int64_t tiles_x = (P.nx + RTX - 1) / RTX;
-        const int64_t ty = lt / tiles_x, tx = lt - ty * tiles_x;
-        if (kind == 0 && (flags & kD8Lowest))
-            recv_d8_tile<false, true>(P.z, P.nx, P.ny, P.mc.co_hi, P.mc.cd_hi, flags,
-                                      const_cast<uint8_t*>(P.rb), nullptr, tx * RTX, ty * RTY);
-        else if (kind == 0)
-            recv_d8_tile<false, false>(P.z, P.nx, P.ny, P.mc.co_hi, P.mc.cd_hi, flags,
-                                       const_cast<uint8_t*>(P.rb), nullptr, tx * RTX, ty * RTY);
-        else
-            recv_mfd_tile<true, false>(P.z, P.nx, P.ny, P.mc, flags, const_cast<uint8_t*>(P.rb),
-                                       const_cast<float*>(P.frac), nullptr, tx * RTX, ty * RTY);
+        int64_t x0, y0;
+        const Prob& P = probs[batch_tile(prefix, nprob, w, probs, x0, y0)];
+        recv_mfd_tile<true, false>(P.z, P.nx, P.ny, P.mc, flags, const_cast<uint8_t*>(P.rb),
+                                   const_cast<float*>(P.frac), nullptr, x0, y0);
         __syncthreads();
     }
 }
@@ -697,14 +793,21 @@ cudaError_t launch_receivers_d8(const float* z, int64_t nx, int64_t ny, double d
         return d4 ? launch_d8_tma<false, true>(map, nx, ny, co, cd, flags, dir, s)
                   : launch_d8_tma<false, false>(map, nx, ny, co, cd, flags, dir, s);
     }
-    if (indeg && lowest)
-        k_receivers_d8<true, true><<<grid, RNT, 0, s>>>(z, nx, ny, co, cd, flags, dir, indeg);
-    else if (indeg)
-        k_receivers_d8<true, false><<<grid, RNT, 0, s>>>(z, nx, ny, co, cd, flags, dir, indeg);
-    else if (lowest)
-        k_receivers_d8<false, true><<<grid, RNT, 0, s>>>(z, nx, ny, co, cd, flags, dir, nullptr);
-    else
-        k_receivers_d8<false, false><<<grid, RNT, 0, s>>>(z, nx, ny, co, cd, flags, dir, nullptr);
+    if (indeg) {
+        if (lowest) k_receivers_d8_indeg<true><<<grid, RNT, 0, s>>>(z, nx, ny, co, cd, flags, dir, indeg);
+        else k_receivers_d8_indeg<false><<<grid, RNT, 0, s>>>(z, nx, ny, co, cd, flags, dir, indeg);
+        return cudaGetLastError();
+    }
+    const int64_t tiles = ((nx + RTX - 1) / RTX) * ((ny + kStrip - 1) / kStrip);
+    const unsigned wgrid = (unsigned)((tiles + RNT / 32 - 1) / (RNT / 32));
+    auto run = [&](auto low, auto d4) {
+        k_receivers_d8<decltype(low)::value, decltype(d4)::value>
+            <<<wgrid, RNT, 0, s>>>(z, nx, ny, co, cd, flags, dir, tiles);
+    };
+    if (lowest && (flags & kD4)) run(std::true_type{}, std::true_type{});
+    else if (lowest) run(std::true_type{}, std::false_type{});
+    else if (flags & kD4) run(std::false_type{}, std::true_type{});
+    else run(std::false_type{}, std::false_type{});
     return cudaGetLastError();
 }
 
@@ -754,7 +857,12 @@ cudaError_t launch_mfd_fractions(const float* z, const uint8_t* mask, int64_t nx
 
 cudaError_t launch_receivers_batch(int kind, const Prob* probs, const int64_t* prefix, int nprob,
                                    uint32_t flags, EngineGlobals* G, int grid, cudaStream_t s) {
-    k_receivers_batch<<<grid, RNT, 0, s>>>(kind, probs, prefix, nprob, flags, G);
+    const bool low = flags & kD8Lowest, d4 = flags & kD4;
+    if (kind != 0) k_receivers_batch_mfd<<<grid, RNT, 0, s>>>(probs, prefix, nprob, flags, G);
+    else if (low && d4) k_receivers_batch_d8<true, true><<<grid, RNT, 0, s>>>(probs, prefix, nprob, flags);
+    else if (low) k_receivers_batch_d8<true, false><<<grid, RNT, 0, s>>>(probs, prefix, nprob, flags);
+    else if (d4) k_receivers_batch_d8<false, true><<<grid, RNT, 0, s>>>(probs, prefix, nprob, flags);
+    else k_receivers_batch_d8<false, false><<<grid, RNT, 0, s>>>(probs, prefix, nprob, flags);
     return cudaGetLastError();
 }
 
