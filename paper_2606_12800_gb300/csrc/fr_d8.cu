@@ -5,17 +5,18 @@
 // paper's per-subdomain high-to-low solve (Sec. 2.4), with overlapping
 // subdomains.  An inner cell is final unless its upstream basin reaches
 // outside the extended region ("global"); on the synthetic fractal DEMs a
-// 4-cell halo leaves about 0.03 % of the cells global, which the walker kernel
-// of fr_engine.cuh then finishes.  Halo cells are solved only to feed the
+// 4-cell halo leaves about 0.03 % of the cells global, which the global
+// phase then finishes.  Halo cells are solved only to feed the
 // inner ones and are not written.
 //
 // Solve: every cell waits for all its donors.  A cell's packed word (arrival
 // count, donors' area sum) starts at its preset; each donor, once final, adds
 // its local area with one shared-memory atomic.  The cells without donors
 // (leaves, two thirds of a rough DEM) are final at once and arrive in one
-// parallel pass; the receivers they complete form a list, and walkers drain
-// it: a walker finalises its cell, arrives at the receiver, and continues
-// with the receiver if it arrived last ("last arriver continues").  No
+// parallel pass that waits for no sum; the receivers they complete, found by a
+// scan behind it, form a list, and walkers drain it, each warp its share: a
+// walker finalises its cell, arrives at the receiver, and continues with the
+// receiver if it arrived last ("last arriver continues").  No
 // block barrier separates the cells of a chain, each cell is visited once, and
 // a cell's two-float value is pulled from its final donors in fixed code
 // order (deterministic sums; exact 16-bit local areas).  The visiting order
@@ -24,12 +25,22 @@
 // outside the region (and cells on a routing cycle) stay unfinished; the inner
 // ones are listed as global.
 //
-// Tiles away from the grid boundary take a vector path: code and rain rows are
-// copied asynchronously (cp.async) in one batch, and the donor masks and
-// arrival counts of four consecutive cells are computed together on packed
-// bytes (a byte-permute builds each neighbour vector, an exact zero-byte test
-// compares four codes at once).  Tiles touching the boundary take a scalar
-// path with bounds tests.
+// Tiles away from the grid boundary whose rows are aligned copy their code and
+// rain rows asynchronously (cp.async) in one batch; the others read them byte by
+// byte, with the codes that point off the grid taken out.  From there on all
+// tiles are alike: the donor masks and arrival counts of four consecutive cells
+// are computed together on packed bytes (codes turned into one bit each, so a
+// donor test is a shift and a mask for four cells).  Cells off the grid have no
+// donors and no receiver: they are final at once and nobody reads them.
+//
+// What bounds it: with water the walk, half of a tile's 34 K cycles, a chain of
+// shared-memory latencies per cell; areas alone, instruction issue.  32768^2,
+// areas: 5.90 ms with eight comparisons per donor mask, a shared hand-out counter
+// and leaf arrivals that waited for their sums, 4.80 ms now.  4096^2, water and
+// areas: 260 -> 228 us; 1537x2603, unaligned: 108 us with a byte-wise solve for
+// such tiles, 75 us now; a batch of 32 clips 504 -> 386 us.  A walker that goes
+// on to a receiver without other donors with no arrival, its sum in registers,
+// was slower (242 us): the lanes of a warp then take one of two ways per step.
 #include <cuda/atomic>
 
 #include "fr_engine.cuh"
@@ -75,10 +86,13 @@ struct SmemD8 {
     alignas(16) uint32_t pk[NR];                  // packed arrivals / donors' area
     alignas(16) uint8_t code[NR];                 // receiver codes of region + ring, padded rows
     alignas(16) uint8_t dm[W ? NR : 16];          // donor masks (value pulls)
-    uint16_t queue[Gm::NE];                       // ready list: cells whose donors (all leaves) finished in the
+    union {
+        alignas(16) uint16_t queue[Gm::NE];       // ready list: cells whose donors (all leaves) finished in the
                                                   // leaf pass; after the walk, the inner tile's unfinished cells
+        uint8_t hot[NR];                          // before that: receiver bit of each cell (1 << code, else 0)
+    };
+    int off[8];                                   // index offset of each code
     int qtail;                                    // its length
-    int head;                                     // next entry to hand out
     int nglob;                                    // unfinished inner cells listed in queue after the walk
     unsigned long long gbase;
     unsigned int done, sinks;  // block sums of the publish step (at most 2^16 and NE)
@@ -105,25 +119,6 @@ __device__ __forceinline__ void push4(S_& S, const int (&cq)[4]) {
         if (cq[q] >= 0) S.queue[pos++] = (uint16_t)cq[q];
 }
 
-// Warp-aggregated append of up to four cells per lane to the ready list (all
-// lanes call; the scalar path).
-template <class S_>
-__device__ __forceinline__ void push_cells(S_& S, int n, const int (&cells)[4]) {
-    const unsigned lane = threadIdx.x & 31u;
-    int incl = n;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if ((int)lane >= o) incl += v;
-    }
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    if (!total) return;
-    int base = 0;
-    if (lane == 31) base = atomicAdd(&S.qtail, total);
-    base = __shfl_sync(0xffffffffu, base, 31) + incl - n;
-    for (int q = 0; q < n; ++q) S.queue[base + q] = (uint16_t)cells[q];
-}
-
 // Per-byte population count.
 __device__ __forceinline__ uint32_t popc_bytes(uint32_t x) {
     x = x - ((x >> 1) & 0x55555555u);
@@ -142,18 +137,14 @@ __device__ __forceinline__ Row3 row3(const uint8_t* row, int w1) {
     return {__byte_perm(a, b, 0x6543), b, __byte_perm(b, d, 0x4321)};
 }
 
-// Neighbour vector of code k from the up / mid / down rows.
-__device__ __forceinline__ uint32_t nbr(const Row3& up, const Row3& mid, const Row3& dn, int k) {
-    switch (k) {
-        case 0: return mid.r;  // E
-        case 1: return up.c;   // N
-        case 2: return mid.l;  // W
-        case 3: return dn.c;   // S
-        case 4: return up.r;   // NE
-        case 5: return up.l;   // NW
-        case 6: return dn.l;   // SW
-        default: return dn.r;  // SE
-    }
+// 1 << code in each byte of x that holds a code 0..7, 0 in the others: a byte
+// permutation looks the bits up, its selectors the codes' nibbles.
+__device__ __forceinline__ uint32_t hot_bytes(uint32_t x) {
+    const uint32_t n = x & 0x0F0F0F0Fu;
+    const uint32_t sel = __byte_perm(n | (n >> 4), 0u, 0x4420);
+    uint32_t ok;  // 0xFF where the byte is a code: prmt with a selector's top bit set spreads the sign
+    asm("prmt.b32 %0, %1, 0, 0xBA98;" : "=r"(ok) : "r"(zero_bytes(x & 0xF8F8F8F8u)));
+    return __byte_perm(0x08040201u, 0x80402010u, sel) & ok;
 }
 
 __device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
@@ -216,8 +207,16 @@ __device__ __forceinline__ int batch_problem(const int64_t* __restrict__ prefix,
     return lo;
 }
 
+// Blocks per SM that the registers leave room for (three for areas alone: 128x64
+// tiles fill the shared memory with as many, and 40 registers instead of 32 took
+// 5.1 ms of a 32768^2 DEM to 4.8).
+template <class Gm, bool W>
+constexpr int d8_blocks() {
+    return W ? (Gm::TX >= 96 ? 2 : 4) : 3;
+}
+
 template <class Gm, bool W, bool AREA, bool BATCH>
-__global__ void __launch_bounds__(Gm::NT) k_local_d8(Prob Pone, EngineGlobals* G,
+__global__ void __launch_bounds__(Gm::NT, d8_blocks<Gm, W>()) k_local_d8(Prob Pone, EngineGlobals* G,
                                                   const Prob* __restrict__ probs,
                                                   const int64_t* __restrict__ prefix, int nprob) {
     constexpr int TX = Gm::TX, TY = Gm::TY, H = Gm::H, EX = Gm::EX, EY = Gm::EY, NE = Gm::NE;
@@ -248,25 +247,18 @@ __global__ void __launch_bounds__(Gm::NT) k_local_d8(Prob Pone, EngineGlobals* G
     // a region cell's packed word starts at its preset (9 - donors) and each donor
     // adds one arrival; the add that completes the count to 9 finalises the cell.
     // Ring cells start at zero and get at most three arrivals, so they never
-    // finish.  The vector path stores the presets after this barrier and zeroes
-    // only the ring here; the scalar path adds the presets atomically, in any
-    // order with the arrivals, onto a zeroed array.
-    if (vec) {
-        for (int i = tid; i < 2 * CP + 2 * EY; i += NT8) {
-            const int r = i < 2 * CP ? (i < CP ? i : (RY - 1) * CP + i - CP)
-                                     : (i - 2 * CP < EY ? (i - 2 * CP + 1) * CP + 3
-                                                        : (i - 2 * CP - EY + 1) * CP + EX + 4);
-            S.pk[r] = 0u;
-        }
-    } else {
-        for (int i = tid; i < Sm::NR / 4; i += NT8) reinterpret_cast<uint4*>(S.pk)[i] = make_uint4(0, 0, 0, 0);
+    // finish.
+    for (int i = tid; i < 2 * CP + 2 * EY; i += NT8) {
+        const int r = i < 2 * CP ? (i < CP ? i : (RY - 1) * CP + i - CP)
+                                 : (i - 2 * CP < EY ? (i - 2 * CP + 1) * CP + 3
+                                                    : (i - 2 * CP - EY + 1) * CP + EX + 4);
+        S.pk[r] = 0u;
     }
+    if (tid < 8) S.off[tid] = offy(tid) * CP + offx(tid);
     if (tid == 0) {
         S.qtail = 0;
-        S.head = 0;
         S.nglob = 0;
     }
-
     if (vec) {
         // ---- asynchronous copies: code rows (8-byte chunks; byte b <-> grid
         // x = x0 - H - 4 + b) and rain rows (16-byte chunks)
@@ -286,163 +278,175 @@ __global__ void __launch_bounds__(Gm::NT) k_local_d8(Prob Pone, EngineGlobals* G
             }
         }
         cp_async_wait_all();
-        __syncthreads();
-        // ---- donor masks and presets (four cells per thread step, plain
-        // stores); the leaves (no donors: final at once) and their receivers'
-        // codes are kept in registers
-        constexpr int NG = (NE / 4 + NT8 - 1) / NT8;
-        static_assert(4 * NG <= 32, "leaf bits of a thread fit one word");
-        uint32_t leaves = 0;       // bit 4 * it + q
-        uint32_t lcode[NG];        // the four codes of group it
-#pragma unroll
-        for (int it = 0; it < NG; ++it) {
-            const int gq = it * NT8 + tid;
-            lcode[it] = 0;
-            if (gq < NE / 4) {
-                const int ey = gq / (EX / 4), ex = (gq - ey * (EX / 4)) * 4;
-                const int w1 = (ex + 4) >> 2;
-                const Row3 up = row3(S.code + ey * CP, w1);
-                const Row3 mid = row3(S.code + (ey + 1) * CP, w1);
-                const Row3 dn = row3(S.code + (ey + 2) * CP, w1);
-                uint32_t dmf = 0;
-#pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    dmf |= zero_bytes(nbr(up, mid, dn, k) ^ (0x01010101u * (uint32_t)opp(k))) >> (7 - k);
-                const uint32_t wait = 0x09090909u - popc_bytes(dmf);  // kPkDone - donors
-                const int r = (ey + 1) * CP + ex + 4;
-                *reinterpret_cast<uint4*>(S.pk + r) =
-                    make_uint4((wait & 0xFFu) << 20, ((wait >> 8) & 0xFFu) << 20,
-                               ((wait >> 16) & 0xFFu) << 20, (wait >> 24) << 20);
-                if constexpr (W) {
-                    *reinterpret_cast<uint32_t*>(S.dm + r) = dmf;
-                    if (!P.init) *reinterpret_cast<float4*>(S.vhi + r) = make_float4(1.f, 1.f, 1.f, 1.f);
-                    *reinterpret_cast<float4*>(S.vlo + r) = make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-                const uint32_t z = zero_bytes(dmf);  // 0x80 per leaf
-                leaves |= (((z >> 7) & 1u) | ((z >> 14) & 2u) | ((z >> 21) & 4u) | ((z >> 28) & 8u)) << (4 * it);
-                lcode[it] = mid.c;
-            }
-        }
-        __syncthreads();
-        // ---- the leaves arrive at their receivers; a receiver completed here
-        // (its last donor was a leaf) goes to the ready list
-#pragma unroll
-        for (int it = 0; it < NG; ++it) {
-            const int gq = it * NT8 + tid;
-            int cq[4] = {-1, -1, -1, -1};
-            const uint32_t lb = (leaves >> (4 * it)) & 0xFu;
-            if (lb) {
-                const int ey = gq / (EX / 4), ex = (gq - ey * (EX / 4)) * 4;
-                const int r = (ey + 1) * CP + ex + 4;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const uint32_t k = (lcode[it] >> (8 * q)) & 0xFFu;
-                    if (!((lb >> q) & 1u) || k >= 8) continue;
-                    const int t = r + q + offy((int)k) * CP + offx((int)k);
-                    const uint32_t add = kPkArrive | 1u;
-                    if (((atomicAdd(&S.pk[t], add) + add) >> 20) == kPkDone) cq[q] = t;
-                }
-            }
-            push4(S, cq);
-        }
     } else {
-        // ---- scalar path (tiles touching the grid boundary)
-        // codes without a receiver in the grid become kNoRecv unless they are
-        // FR_SINK, so that kSink marks exactly the routing bytes FR_SINK (the
-        // mass balance's sinks), as on the vector path, which keeps the bytes
-        for (int i = tid; i < RY * CP; i += NT8) {
-            const int ry = i / CP, rx = i - ry * CP - 3;
-            uint8_t code = kNoRecv;
-            if (rx >= gx_lo && rx < gx_hi && ry >= gy_lo && ry < gy_hi) {
-                code = rd_rb(P, (oy + ry) * P.nx + (ox + rx));
-                if (code < 8) {
-                    const int xr = rx + offx(code), yr = ry + offy(code);
-                    if (xr < gx_lo || xr >= gx_hi || yr < gy_lo || yr >= gy_hi) code = kNoRecv;
-                } else if (code != kSink) {
-                    code = kNoRecv;
-                }
-            }
-            S.code[i] = code;
-        }
-        __syncthreads();
-        for (int c0 = 0; c0 < NE; c0 += NT8) {
-            const int c = c0 + tid;
-            int cells[4];
-            int n = 0;
-            if (c < NE) {
-                const int ey = c / EX, ex = c - ey * EX;
-                const int rx = ex + 1, ry = ey + 1;
-                const int r = ry * CP + rx + 3;
-                uint32_t dm = 0;
-                if (rx >= gx_lo && rx < gx_hi && ry >= gy_lo && ry < gy_hi) {
+        // ---- a warp per row, the loads of two rows issued before the first is
+        // used.  Codes without a receiver in the grid become kNoRecv unless they
+        // are FR_SINK, so that kSink marks exactly the routing bytes FR_SINK (the
+        // mass balance's sinks), as on the other path, which keeps the bytes.
+        // (one row where the occupancy rests on 32 registers)
+        constexpr int C = (CP + 31) / 32, NW8 = NT8 / 32, U = W && TX >= 96 ? 2 : 1;
+        const int warp = tid >> 5, lane = tid & 31;
+        const bool inside = gx_lo == 0 && gy_lo == 0 && gx_hi == EX + 2 && gy_hi == RY;
+        for (int r0 = warp; r0 < RY; r0 += U * NW8) {
+            uint8_t cd[U][C];
+            float rn[U][C];
 #pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        dm |= (uint32_t)(S.code[r + offy(k) * CP + offx(k)] == (uint8_t)opp(k)) << k;
-                    if constexpr (W) {
-                        const int64_t gi = (oy + ry) * P.nx + (ox + rx);
-                        S.vhi[r] = P.init ? rd_in(P.init, P, gi, 8) : 1.0f;
-                        S.vlo[r] = 0.0f;
-                        S.dm[r] = (uint8_t)dm;
-                    }
-                    const uint32_t pre = (kPkDone - (uint32_t)__popc(dm)) << 20;
-                    const uint32_t old = atomicAdd(&S.pk[r], pre);
-                    if (((old + pre) >> 20) == kPkDone) {
-                        if (dm) {
-                            cells[n++] = r;
-                        } else {
-                            const uint32_t k = S.code[r];
-                            if (k < 8) {
-                                const int t = r + offy((int)k) * CP + offx((int)k);
-                                const uint32_t add = kPkArrive | 1u;
-                                if (((atomicAdd(&S.pk[t], add) + add) >> 20) == kPkDone) cells[n++] = t;
-                            }
-                        }
+            for (int u = 0; u < U; ++u) {
+                const int ry = r0 + u * NW8;
+                const int64_t row = (oy + ry) * P.nx + ox;
+                const bool in_y = ry < RY && (inside || (ry >= gy_lo && ry < gy_hi));
+#pragma unroll
+                for (int q = 0; q < C; ++q) {
+                    const int rx = lane + 32 * q - 3;
+                    cd[u][q] = kNoRecv;
+                    rn[u][q] = 1.0f;
+                    if (in_y && rx >= gx_lo && rx < gx_hi) {
+                        cd[u][q] = rd_rb(P, row + rx);
+                        if (W && P.init) rn[u][q] = rd_in(P.init, P, row + rx, 8);
                     }
                 }
-                // outside the grid: no preset, no donors; never final
             }
-            push_cells(S, n, cells);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int ry = r0 + u * NW8;
+                if (ry >= RY) break;
+#pragma unroll
+                for (int q = 0; q < C; ++q) {
+                    const int b = lane + 32 * q, rx = b - 3;
+                    if (b >= CP) continue;
+                    uint32_t code = cd[u][q];
+                    if (code < 8) {
+                        const int xr = rx + offx((int)code), yr = ry + offy((int)code);
+                        if (xr < gx_lo || xr >= gx_hi || yr < gy_lo || yr >= gy_hi) code = kNoRecv;
+                    } else if (code != kSink) {
+                        code = kNoRecv;
+                    }
+                    S.code[ry * CP + b] = (uint8_t)code;
+                    if constexpr (W) {
+                        if (P.init) S.vhi[ry * CP + b] = rn[u][q];
+                    }
+                }
+            }
         }
+    }
+    __syncthreads();
+    for (int i = tid; i < Sm::NR / 4; i += NT8)
+        reinterpret_cast<uint32_t*>(S.hot)[i] = hot_bytes(reinterpret_cast<const uint32_t*>(S.code)[i]);
+    __syncthreads();
+    // ---- donor masks and presets (four cells per thread step); the leaves (no
+    // donors: final at once) are kept in registers
+    constexpr int NG = (NE / 4 + NT8 - 1) / NT8;
+    static_assert(4 * NG <= 32, "leaf bits of a thread fit one word");
+    uint32_t leaves = 0;  // bit 4 * it + q
+#pragma unroll
+    for (int it = 0; it < NG; ++it) {
+        const int gq = it * NT8 + tid;
+        if (gq < NE / 4) {
+            const int ey = gq / (EX / 4), ex = (gq - ey * (EX / 4)) * 4;
+            const int w1 = (ex + 4) >> 2;
+            const Row3 up = row3(S.hot + ey * CP, w1);
+            const Row3 mid = row3(S.hot + (ey + 1) * CP, w1);
+            const Row3 dn = row3(S.hot + (ey + 2) * CP, w1);
+            // the donor in direction k has its bit opp(k) = k ^ 2 set
+            uint32_t dmf = ((mid.r >> 2) & 0x01010101u) | ((up.c >> 2) & 0x02020202u);
+            dmf |= ((mid.l << 2) & 0x04040404u) | ((dn.c << 2) & 0x08080808u);
+            dmf |= ((up.r >> 2) & 0x10101010u) | ((up.l >> 2) & 0x20202020u);
+            dmf |= ((dn.l << 2) & 0x40404040u) | ((dn.r << 2) & 0x80808080u);
+            const uint32_t wait = 0x09090909u - popc_bytes(dmf);  // kPkDone - donors
+            const int r = (ey + 1) * CP + ex + 4;
+            *reinterpret_cast<uint4*>(S.pk + r) =
+                make_uint4((wait & 0xFFu) << 20, ((wait >> 8) & 0xFFu) << 20,
+                           ((wait >> 16) & 0xFFu) << 20, (wait >> 24) << 20);
+            if constexpr (W) {
+                *reinterpret_cast<uint32_t*>(S.dm + r) = dmf;
+                if (!P.init) *reinterpret_cast<float4*>(S.vhi + r) = make_float4(1.f, 1.f, 1.f, 1.f);
+                *reinterpret_cast<float4*>(S.vlo + r) = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            const uint32_t z = zero_bytes(dmf);  // 0x80 per leaf
+            leaves |= (((z >> 7) & 1u) | ((z >> 14) & 2u) | ((z >> 21) & 4u) | ((z >> 28) & 8u)) << (4 * it);
+        }
+    }
+    __syncthreads();
+    // ---- the leaves arrive at their receivers (nobody waits for the sums)
+#pragma unroll
+    for (int it = 0; it < NG; ++it) {
+        const uint32_t lb = (leaves >> (4 * it)) & 0xFu;
+        if (lb) {
+            const int gq = it * NT8 + tid;
+            const int ey = gq / (EX / 4), ex = (gq - ey * (EX / 4)) * 4;
+            const int r = (ey + 1) * CP + ex + 4;
+            const uint32_t lcode = *reinterpret_cast<const uint32_t*>(S.code + r);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t k = (lcode >> (8 * q)) & 0xFFu;
+                if (((lb >> q) & 1u) && k < 8) atomicAdd(&S.pk[r + q + S.off[k]], kPkArrive | 1u);
+            }
+        }
+    }
+    __syncthreads();
+    // ---- cells whose donors were all leaves: final, not leaves themselves
+#pragma unroll
+    for (int it = 0; it < NG; ++it) {
+        const int gq = it * NT8 + tid;
+        int cq[4] = {-1, -1, -1, -1};
+        if (gq < NE / 4) {
+            const int ey = gq / (EX / 4), ex = (gq - ey * (EX / 4)) * 4;
+            const int r = (ey + 1) * CP + ex + 4;
+            const uint4 p = *reinterpret_cast<const uint4*>(S.pk + r);
+            const uint32_t lb = leaves >> (4 * it);
+            if (pk_final(p.x) && !(lb & 1u)) cq[0] = r;
+            if (pk_final(p.y) && !(lb & 2u)) cq[1] = r + 1;
+            if (pk_final(p.z) && !(lb & 4u)) cq[2] = r + 2;
+            if (pk_final(p.w) && !(lb & 8u)) cq[3] = r + 3;
+        }
+        push4(S, cq);
     }
     __syncthreads();
 
     // ---- walkers: a lane finalises a cell, adds it to its receiver's packed
     // word and continues with the receiver when it arrived last; otherwise it
-    // takes the next start (warp-aggregated hand-out from the block's list)
+    // takes the next start of its warp's share of the list
     {
         const unsigned lane = tid & 31u;
         const unsigned below = (1u << lane) - 1u;
         const int nst = S.qtail;
-        int c = -1;        // ring index of the cell being finalised
-        uint32_t a = 0;    // its local area
-        bool more = true;  // warp-uniform: list entries may be left
+        constexpr int NW8 = NT8 / 32;
+        int next_start = nst * (tid >> 5) / NW8;  // warp-uniform
+        const int end = nst * ((tid >> 5) + 1) / NW8;
+        int c = -1;      // ring index of the cell being finalised
+        uint32_t a = 0;  // its local area
         for (;;) {
-            if (more) {
+            if (next_start < end) {
                 const unsigned idle = __ballot_sync(0xffffffffu, c < 0);
-                if (idle) {
-                    const int leader = __ffs(idle) - 1;
-                    int base = 0;
-                    if ((int)lane == leader) base = atomicAdd(&S.head, __popc(idle));
-                    base = __shfl_sync(0xffffffffu, base, leader);
-                    if (c < 0) {
-                        const int i = base + __popc(idle & below);
-                        if (i < nst) {
-                            c = S.queue[i];
-                            a = 1u + (S.pk[c] & kPkArea);  // final: all donors arrived
-                        }
+                if (c < 0) {
+                    const int i = next_start + __popc(idle & below);
+                    if (i < end) {
+                        c = S.queue[i];
+                        a = 1u + (S.pk[c] & kPkArea);  // final: all donors arrived
                     }
-                    if (base + __popc(idle) >= nst) more = false;
                 }
+                next_start += __popc(idle);
             }
             if (!__any_sync(0xffffffffu, c >= 0)) break;
             if (c < 0) continue;
             if constexpr (W) {
                 // the cell's donors are final: pull their values in ascending code order
                 df v = {S.vhi[c], S.vlo[c]};
-                for (uint32_t m = S.dm[c]; m; m &= m - 1) {
-                    const int k = __ffs(m) - 1;
-                    const int j = c + offy(k) * CP + offx(k);
-                    v = df_add(v, df{S.vhi[j], S.vlo[j]});
+                uint32_t m = S.dm[c];
+                if constexpr (TX >= 96) {
+                    // the next donor's index runs ahead of the addition
+                    int j = c + S.off[(__ffs(m) - 1) & 7];
+                    while (m) {
+                        const df u = {S.vhi[j], S.vlo[j]};
+                        m &= m - 1;
+                        j = c + S.off[(__ffs(m) - 1) & 7];
+                        v = df_add(v, u);
+                    }
+                } else {  // 32 registers: no room for it
+                    for (; m; m &= m - 1) {
+                        const int j = c + S.off[__ffs(m) - 1];
+                        v = df_add(v, df{S.vhi[j], S.vlo[j]});
+                    }
                 }
                 S.vhi[c] = v.hi;
                 S.vlo[c] = v.lo;
@@ -450,7 +454,7 @@ __global__ void __launch_bounds__(Gm::NT) k_local_d8(Prob Pone, EngineGlobals* G
             const uint32_t k = S.code[c];
             int next = -1;
             if (k < 8) {
-                const int t = c + offy((int)k) * CP + offx((int)k);
+                const int t = c + S.off[k];
                 const uint32_t add = kPkArrive | a;
                 uint32_t old;
                 if constexpr (W) {
@@ -476,10 +480,10 @@ __global__ void __launch_bounds__(Gm::NT) k_local_d8(Prob Pone, EngineGlobals* G
     // routing byte is FR_SINK are summed for the mass balance (the global
     // phase's cells are summed there from the global-cell bits).
     // Per-thread counts: at most 16 inner cells a thread, areas below 2^16.
-    // Whole vector tiles count their finished cells as the inner cells less the
-    // listed ones instead.
+    // Tiles that lie in the grid count their finished cells as the inner cells less
+    // the listed ones instead.
     uint32_t done = 0, sinks = 0;
-    const bool whole = vec && x0 + TX <= P.nx && y0 + TY <= P.ny;
+    const bool whole = x0 + TX <= P.nx && y0 + TY <= P.ny;
     auto need_lo_of = [&](int r, int lx, int ly) -> bool {
         // a cell's trailing word is pulled later when its receiver leaves the
         // inner tile (another tile may list it as global) or is global here
@@ -522,16 +526,31 @@ __global__ void __launch_bounds__(Gm::NT) k_local_d8(Prob Pone, EngineGlobals* G
             }
             const int64_t gi = (y0 + ly) * P.nx + x0 + lx;
             if constexpr (W) {
-                *reinterpret_cast<float4*>(P.out_hi + gi) = *reinterpret_cast<const float4*>(S.vhi + r);
+                const float4 v = *reinterpret_cast<const float4*>(S.vhi + r);
+                if (vec) {
+                    *reinterpret_cast<float4*>(P.out_hi + gi) = v;
+                } else {
+                    P.out_hi[gi] = v.x;
+                    P.out_hi[gi + 1] = v.y;
+                    P.out_hi[gi + 2] = v.z;
+                    P.out_hi[gi + 3] = v.w;
+                }
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
                     if (P.lo_full || need_lo_of(r + q, lx + q, ly))
                         wr_f(P.out_lo, P, gi + q, S.vlo[r + q], 28);
             }
             if constexpr (AREA) {
-                ulonglong2* out = reinterpret_cast<ulonglong2*>(P.area + gi);
-                out[0] = make_ulonglong2(1u + (p4.x & kPkArea), 1u + (p4.y & kPkArea));
-                out[1] = make_ulonglong2(1u + (p4.z & kPkArea), 1u + (p4.w & kPkArea));
+                if (vec) {
+                    ulonglong2* out = reinterpret_cast<ulonglong2*>(P.area + gi);
+                    out[0] = make_ulonglong2(1u + (p4.x & kPkArea), 1u + (p4.y & kPkArea));
+                    out[1] = make_ulonglong2(1u + (p4.z & kPkArea), 1u + (p4.w & kPkArea));
+                } else {
+                    P.area[gi] = 1u + (p4.x & kPkArea);
+                    P.area[gi + 1] = 1u + (p4.y & kPkArea);
+                    P.area[gi + 2] = 1u + (p4.z & kPkArea);
+                    P.area[gi + 3] = 1u + (p4.w & kPkArea);
+                }
                 if constexpr (!BATCH) {
                     // byte q of sk is 1 where routing byte q is FR_SINK; the areas
                     // are 1 + the 16-bit donor sums: a count plus two 16x8-bit dot
