@@ -144,19 +144,17 @@ Prob base_prob(const fr_routing* R, char* ws, bool with_water = false) {
     P.glist_cap = R->nx * R->ny;
     P.out_lo = reinterpret_cast<float*>(ws + L.lo);
     // the skeleton solve's scratch shares the global-cell list's region (the
-    // list itself is read only by the cell walkers): tile list, walker
-    // starts, dependency slots
+    // list itself is read only by the cell walkers): walker starts, dependency
+    // slots
     P.skel_min = ~0ull;
     if (R->kind == FR_ROUTING_D8) {
         const int side = skel_side(with_water);
         const int64_t n = R->nx * R->ny, st = skel_tiles(R->nx, R->ny, side);
-        const size_t o_starts = align256((size_t)st * 4);
-        const size_t o_pool = o_starts + align256((size_t)st * (4 * side - 4) * 8);
+        const size_t o_pool = align256((size_t)st * (4 * side - 4) * 8);
         const size_t need = o_pool + (size_t)st * skel_pool(side) * 2;
         if (need <= (size_t)n * 8 && !(R->flags & FR_GLOBAL_WALKERS)) {
             char* base = ws + L.glist;
-            P.sktiles = reinterpret_cast<uint32_t*>(base);
-            P.skstarts = reinterpret_cast<unsigned long long*>(base + o_starts);
+            P.skstarts = reinterpret_cast<unsigned long long*>(base);
             P.skpool = reinterpret_cast<uint16_t*>(base + o_pool);
             const double share = (double)n * kSkelShare;
             P.skel_min = (R->flags & FR_GLOBAL_SKELETON) ? 0ull

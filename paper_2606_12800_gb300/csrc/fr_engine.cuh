@@ -824,13 +824,16 @@ cudaError_t launch_global(const Prob* probs, const Prob& single, EngineGlobals* 
     unsigned long long poll_max = (unsigned long long)gp * 256 * kPollCells;
     unsigned long long limit = wait_limit_ns();
     void* args[] = {(void*)&pp, (void*)&one, (void*)&G, (void*)&total, (void*)&poll_max, (void*)&limit};
-    e = cudaLaunchCooperativeKernel((const void*)k_global_poll<M, W, AREA>, dim3(gp), dim3(256), args, 0, s);
+    // no more blocks than the grid could fill with global cells
+    const unsigned long long most = (total_cells + 255) / 256;
+    const unsigned blocks = most < (unsigned long long)gp ? (unsigned)(most ? most : 1) : (unsigned)gp;
+    e = cudaLaunchCooperativeKernel((const void*)k_global_poll<M, W, AREA>, dim3(blocks), dim3(256), args, 0, s);
     if (e != cudaSuccess || total_cells <= poll_max) return e;
     if constexpr (M == Mode::FwdD8) {
-        k_global_init<M, W, AREA><<<walker_grid(), 256, 0, s>>>(probs, single, G, poll_max);
+        k_global_init<M, W, AREA><<<walker_grid() / 2, 256, 0, s>>>(probs, single, G, poll_max);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        k_global<M, W, AREA><<<walker_grid(), 256, 0, s>>>(probs, single, G, total_cells, poll_max);
+        k_global<M, W, AREA><<<walker_grid() / 2, 256, 0, s>>>(probs, single, G, total_cells, poll_max);
         return cudaGetLastError();
     } else {
         static int grid_lev[64] = {};

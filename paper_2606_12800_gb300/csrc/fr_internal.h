@@ -46,7 +46,6 @@ struct Prob {
     unsigned long long skel_min;
     uint16_t* skpool;               // dependency slots, skel_pool per skeleton tile
     unsigned long long* skstarts;   // exits that start a skeleton walker
-    uint32_t* sktiles;              // skeleton tiles holding global cells
 };
 
 // Device-wide bookkeeping kept at the start of the workspace; zeroed (with
@@ -64,7 +63,7 @@ struct EngineGlobals {
     unsigned int bar_count;          // grid barrier: blocks arrived
     unsigned int bar_gen;            // grid barrier: generation
     unsigned long long rounds;       // level-synchronous global phase: rounds run (diagnostic)
-    unsigned long long skel_tiles;   // skeleton solve: tiles listed in Prob::sktiles
+    unsigned long long unused;
     unsigned long long sink_area;    // D8 areas: sum of the areas of the FR_SINK cells the local phase finished
     unsigned long long pad[2];
 };

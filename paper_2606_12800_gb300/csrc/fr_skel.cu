@@ -585,46 +585,18 @@ __device__ void walk_pull(S_& S) {
     }
 }
 
-// Tiles holding at least one global cell, listed once per call (one warp per
-// tile reads the tile's rows of the global-cell bits).
-template <bool W>
-__global__ void __launch_bounds__(256) k_skel_tiles(Prob P, EngineGlobals* G, int64_t ntiles) {
-    if (__ldcg(&G->glist_count) < P.skel_min) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x / 32);
-    for (int64_t t = (int64_t)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); t < ntiles; t += warps) {
-        const TileGeo g = tile_geo<W>(P, t);
-        uint32_t any = 0;
-        for (int ly = lane; ly < g.ey; ly += 32) {
-            const int64_t b0 = (g.y0 + ly) * P.nx + g.x0, b1 = b0 + g.ex;  // bits [b0, b1)
-            for (int64_t wd = b0 >> 5; wd <= (b1 - 1) >> 5; ++wd) {
-                uint32_t m = __ldg(P.gbits + wd);
-                const int64_t lo = wd << 5;
-                if (b0 > lo) m &= ~0u << (b0 - lo);
-                if (b1 < lo + 32) m &= (1u << (b1 - lo)) - 1u;
-                any |= m;
-            }
-        }
-        if (__any_sync(0xffffffffu, any != 0) && lane == 0) {
-            const unsigned long long slot = atomicAdd(&G->skel_tiles, 1ull);
-            P.sktiles[slot] = (uint32_t)t;
-        }
-    }
-}
-
 // Pass A: in-tile partial values, exits, entries and dependency lists.
 template <bool W, bool AREA>
-__global__ void __launch_bounds__(SkGeo<W>::NT, SkGeo<W>::kBlocks) k_skel_a(Prob P, EngineGlobals* G) {
+__global__ void __launch_bounds__(SkGeo<W>::NT, SkGeo<W>::kBlocks) k_skel_a(Prob P, EngineGlobals* G,
+                                                                            int64_t ntiles) {
     using Sm = SmemSk<W, AREA>;
     constexpr int SX = Sm::SX, SRX = Sm::SRX, kSkNT = Sm::kSkNT, kSkelPool = Sm::kPool;
     constexpr bool kPush = Sm::kPush;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Sm& S = *reinterpret_cast<Sm*>(smem_raw);
     if (__ldcg(&G->glist_count) < P.skel_min) return;
-    const unsigned long long ntl = __ldcg(&G->skel_tiles);
     const int tid = threadIdx.x;
-    for (unsigned long long it = blockIdx.x; it < ntl; it += gridDim.x) {
-        const int64_t t = (int64_t)__ldcg(P.sktiles + it);
+    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const TileGeo g = tile_geo<W>(P, t);
         __syncthreads();  // the previous tile's shared memory is no longer read
         if (tid == 0) {
@@ -633,6 +605,7 @@ __global__ void __launch_bounds__(SkGeo<W>::NT, SkGeo<W>::kBlocks) k_skel_a(Prob
         }
         load_tile(S, P, g);
         const int ng = S.ng;
+        if (ng == 0) continue;
         // ---- start values: rain (or 1) plus the final values of non-global
         // donors in code order; in-tile global donors counted
         for (int i0 = 0; i0 < ng; i0 += kSkNT) {  // warp-uniform trip count
@@ -993,19 +966,18 @@ __global__ void __launch_bounds__(256) k_skel_walk(Prob P, EngineGlobals* G) {
 // values of the global cells; completion count.
 template <bool W, bool AREA>
 __global__ void __launch_bounds__(SkGeo<W>::NT, SkGeo<W>::kBlocks) k_skel_fix(Prob P, EngineGlobals* G,
-                                                   unsigned long long total_cells) {
+                                                                              int64_t ntiles,
+                                                                              unsigned long long total_cells) {
     using Sm = SmemSk<W, AREA>;
     constexpr int SX = Sm::SX, SRX = Sm::SRX, kSkNT = Sm::kSkNT;
     constexpr bool kPush = Sm::kPush;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Sm& S = *reinterpret_cast<Sm*>(smem_raw);
     if (__ldcg(&G->glist_count) < P.skel_min) return;
-    const unsigned long long ntl = __ldcg(&G->skel_tiles);
     const uint8_t* done_b = reinterpret_cast<const uint8_t*>(P.cnt);
     const int tid = threadIdx.x;
     unsigned long long done = 0;
-    for (unsigned long long it = blockIdx.x; it < ntl; it += gridDim.x) {
-        const int64_t t = (int64_t)__ldcg(P.sktiles + it);
+    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const TileGeo g = tile_geo<W>(P, t);
         __syncthreads();
         if (tid == 0) {
@@ -1014,6 +986,7 @@ __global__ void __launch_bounds__(SkGeo<W>::NT, SkGeo<W>::kBlocks) k_skel_fix(Pr
         }
         load_tile(S, P, g);
         const int ng = S.ng;
+        if (ng == 0) continue;
         // ---- inflow of every entry: the totals of its donors in other tiles
         // (exits, final after pass B), one thread per boundary cell
         const int nb = nboundary(g.ex, g.ey);
@@ -1219,19 +1192,15 @@ cudaError_t launch_skel_t(const Prob& P, EngineGlobals* G, cudaStream_t s) {
     if (!grid_a || !grid_c) return cudaErrorInvalidConfiguration;
     const int64_t ntiles = skel_tiles(P.nx, P.ny, skel_side(W));
     constexpr int kSkNT = SkGeo<W>::NT;
-    int tgrid = (int)((ntiles + 7) / 8);
-    if (tgrid > 16 * 152) tgrid = 16 * 152;
-    if (tgrid < 1) tgrid = 1;
-    k_skel_tiles<W><<<tgrid, 256, 0, s>>>(P, G, ntiles);
+    const unsigned ga = (unsigned)(ntiles < grid_a ? ntiles : grid_a), gc = (unsigned)(ntiles < grid_c ? ntiles : grid_c);
+    k_skel_a<W, AREA><<<ga, kSkNT, sm, s>>>(P, G, ntiles);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_skel_a<W, AREA><<<grid_a, kSkNT, sm, s>>>(P, G);
+    const int64_t wg = (P.nx * P.ny + 255) / 256;
+    k_skel_walk<W, AREA><<<(unsigned)(wg < walker_grid() / 2 ? wg : walker_grid() / 2), 256, 0, s>>>(P, G);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_skel_walk<W, AREA><<<walker_grid() / 2, 256, 0, s>>>(P, G);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_skel_fix<W, AREA><<<grid_c, kSkNT, sm, s>>>(P, G, (unsigned long long)(P.nx * P.ny));
+    k_skel_fix<W, AREA><<<gc, kSkNT, sm, s>>>(P, G, ntiles, (unsigned long long)(P.nx * P.ny));
     return cudaGetLastError();
 }
 
