@@ -642,6 +642,14 @@ cudaError_t launch_d8_forward(bool want_w, bool want_area, const Prob& P, Engine
     // alone need 5 bytes, which leaves room for 128x64 tiles (1.20x, three
     // blocks per SM).  Each measured fastest among 64x32 ... 128x96 for its
     // case (with values: 128x32 and 64x64 were 5 % slower at 4096^2).
+    // Grids with fewer 96x48 tiles than SMs take 64x32 tiles, whose solve is
+    // shorter: with water 160^2 18.5 -> 14.2 us, 768^2 20.7 -> 18.6, areas alone
+    // 17.0 -> 9.6 and 18.2 -> 12.5 (1024^2, 242 tiles: 26.5 and 27.4, no gain).
+    if (halo_tiles(0, 2, P.nx, P.ny) <= walker_grid() / 8) {
+        if (want_w && want_area) return launch_d8<GeoD8s, true, true>(P, G, s);
+        if (want_w) return launch_d8<GeoD8s, true, false>(P, G, s);
+        return launch_d8<GeoD8s, false, true>(P, G, s);
+    }
     if (want_w && want_area) return launch_d8<GeoD8w, true, true>(P, G, s);
     if (want_w) return launch_d8<GeoD8w, true, false>(P, G, s);
     return launch_d8<D8Geo<kD8TileX, 2 * kD8TileY>, false, true>(P, G, s);

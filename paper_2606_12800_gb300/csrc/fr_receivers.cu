@@ -784,9 +784,11 @@ cudaError_t launch_receivers_d8(const float* z, int64_t nx, int64_t ny, double d
     float co = (float)(1.0 / dx);
     float cd = (float)(1.0 / (std::sqrt(2.0) * dx));
     const bool lowest = flags & kD8Lowest;
-    // codes alone on a TMA-addressable grid: the pipelined persistent kernel
+    // codes alone on a TMA-addressable grid that gives most SMs a tile: the
+    // pipelined persistent kernel (below 2^20 cells the strips are the faster:
+    // 5 to 6 us against 7; 768^2 6.2 and 7.1, 1024^2 7.5 and 7.2, 2048^2 19 and 15)
     CUtensorMap map;
-    if (!indeg && nx * ny >= (int64_t)TTX * TTY && encode_tile_map_f32(&map, z, nx, ny, TBX, TBY)) {
+    if (!indeg && nx * ny >= (int64_t)1 << 20 && encode_tile_map_f32(&map, z, nx, ny, TBX, TBY)) {
         const bool d4 = flags & kD4;
         if (lowest) return d4 ? launch_d8_tma<true, true>(map, nx, ny, co, cd, flags, dir, s)
                               : launch_d8_tma<true, false>(map, nx, ny, co, cd, flags, dir, s);

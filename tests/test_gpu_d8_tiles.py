@@ -1,5 +1,5 @@
 """D8 tile solve: aligned and unaligned tiles, tile edges (96x48 with water,
-128x64 for areas alone, 64x32 in batches) and routing bytes that are no codes."""
+128x64 for areas alone, 64x32 on small grids and in batches) and routing bytes that are no codes."""
 import numpy as np
 import pytest
 
@@ -10,7 +10,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("shape", [(48, 96), (64, 128), (47, 95), (65, 129), (145, 290), (144, 296), (200, 400)])
+@pytest.mark.parametrize("shape", [(48, 96), (64, 128), (47, 95), (65, 129), (145, 290), (144, 296), (200, 400), (1000, 1200)])
 @pytest.mark.parametrize("shift", [0, 1])
 def test_invalid_bytes_have_no_receiver(shape, shift):
     """Any byte above 7 is a cell without a receiver, on every loading path

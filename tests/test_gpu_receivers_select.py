@@ -20,7 +20,7 @@ def _surfaces(ny, nx):
     yield inputs.fractal_dem(ny, nx, beta=2.0, tilt=0.0, seed=5) - np.float32(500.0), 30.0
 
 
-@pytest.mark.parametrize("shape", [(3, 5), (4, 127), (5, 129), (9, 257), (64, 128), (66, 260), (131, 132)])
+@pytest.mark.parametrize("shape", [(3, 5), (4, 127), (5, 129), (9, 257), (64, 128), (66, 260), (131, 132), (1024, 1028)])
 @pytest.mark.parametrize("flags", [0, oracle.EDGE_ROUTE, oracle.D8_LOWEST, oracle.D4 | oracle.EDGE_ROUTE])
 def test_ties_flats_and_underflow(shape, flags):
     from paper_2606_12800_gb300 import api
