@@ -50,7 +50,7 @@
 // of the scattered reads while levels are wide, latency when they are narrow),
 // 66 K cycles per region in all.  8192^2: 5.37 ms forward and 5.38 adjoint with
 // the queue of ready cells that this replaces (270 K warp instructions per 64x64
-// tile at 14 busy lanes), 2.87 and 3.14 ms now.
+// tile at 14 busy lanes), 2.83 and 2.91 ms now.
 #include "fr_engine.cuh"
 
 namespace fr {
@@ -101,7 +101,7 @@ struct SmemHalo {
     int wide, narrow;                   // from level `wide` on at most kHaloMid cells each, from `narrow` 32
     unsigned int ndone;
 };
-constexpr int kHaloMid = 256;
+constexpr int kHaloMid = 512;
 
 // Plane and offset in `edge` of the edge from a cell in direction k.
 __device__ __forceinline__ constexpr int edge_plane(int k) {
@@ -404,8 +404,9 @@ __global__ void __launch_bounds__(kHaloNT, 1) k_local_halo(Prob Pone, EngineGlob
             vi[u].hi = rd_in(P.init, P, gi, 8);
         } else if (!S.dm[c]) {
             // L = sum over sinks of w^2: gbar = 2 w at a sink, 0 elsewhere
-            vi[u].hi = __fmul_rn(2.0f, rd_in(P.wf, P, gi, 9));
-            vi[u].lo = P.wf_lo ? __fmul_rn(2.0f, rd_in(P.wf_lo, P, gi, 10)) : 0.0f;
+            // (doubled below, so that no load is waited for here)
+            vi[u].hi = rd_in(P.wf, P, gi, 9);
+            if (P.wf_lo) vi[u].lo = rd_in(P.wf_lo, P, gi, 10);
         }
     }
     // ---- the levels' cells, packed: a warp per level (two at most) counts,
@@ -478,12 +479,16 @@ __global__ void __launch_bounds__(kHaloNT, 1) k_local_halo(Prob Pone, EngineGlob
         const int c = tid + u * NT;
         if (c >= HaloGeo::NE) break;
         // a cell without dependencies is final: as a sum without terms leaves it
-        if (HM::kAdj && !S.dm[c]) vi[u] = df_norm(vi[u].hi, vi[u].lo);
+        if (HM::kAdj && !S.dm[c]) {
+            if (!P.init) vi[u] = {__fmul_rn(2.0f, vi[u].hi), __fmul_rn(2.0f, vi[u].lo)};
+            vi[u] = df_norm(vi[u].hi, vi[u].lo);
+        }
         S.v[c] = make_float2(vi[u].hi, vi[u].lo);
     }
     __syncthreads();
-    // ---- the levels in order: all warps, then eight, then one as the levels
-    // shrink
+    // ---- the levels in order: all warps, then half of them, then one as
+    // the levels shrink (the barrier among fewer warps is the shorter: halves at 128,
+    // 256, 384 and 512 cells 209, 206, 204 and 203 us at 2048^2)
     auto solve = [&](int c, uint32_t m) {
         float f[8];
         df vv[8];

@@ -456,12 +456,13 @@ __global__ void __launch_bounds__(RNT) k_receivers_mfd(const float* __restrict__
 // Masks and fractions of the slope split.  The weight u = s^p of an edge is the
 // same number whichever of its two cells is asked, and only the higher one
 // gives water along it, so it is computed once per edge: four powers a cell
-// (E, S, SE, SW; 4.4 with the tile's rim), each by a lane that needs it, where
+// (E, S, SE, SW; 4.25 with the tile's rim), each by a lane that needs it, where
 // asking each cell for its lower neighbours runs all eight under masks.  Bound
 // by instruction issue (the power is about 45 operations).  8192^2: masks and
 // fractions 1.61 ms per cell, 1.19 by edges, 1.05 with the shorter power of
-// mfd_pow_normal; fractions of given masks 1.49, 1.16 and 1.02 ms.
-constexpr int WTX = 64, WTY = 16;                     // tile
+// mfd_pow_normal, 1.00 in 64x32 tiles; fractions of given masks 1.49, 1.16, 1.02
+// and 0.97 ms.
+constexpr int WTX = 64, WTY = 32;                     // tile (64x16 1.05 ms, 64x24 and 128x16 1.01)
 constexpr int WZX = WTX + 2, WZY = WTY + 2;           // elevations with a one-cell rim
 constexpr int WEN = WZX * (WTY + 1);                  // edges: rows -1 .. WTY - 1, columns -1 .. WTX
 

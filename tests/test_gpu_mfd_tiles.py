@@ -109,12 +109,13 @@ def _check(ny, nx, make, flags, with_rain):
     np.testing.assert_array_equal(g.cpu().numpy(), _solve(mask, frac, gbar, adjoint=True)[0])
 
 
-@pytest.mark.parametrize("shape", [(15, 63), (16, 64), (17, 65), (18, 66), (33, 129), (1, 70), (70, 1), (2, 2)])
+@pytest.mark.parametrize("shape", [(15, 63), (16, 64), (17, 65), (18, 66), (33, 129), (1, 70), (70, 1), (2, 2),
+                                   (31, 64), (32, 65), (34, 63)])
 @pytest.mark.parametrize("flags", [0, oracle.EDGE_ROUTE])
 @pytest.mark.parametrize("p", [0.5, 1.0, 1.1, 4.5])
 def test_mfd_weights_tile_edges(shape, flags, p):
     """Masks (with and without fractions) bit for bit, fractions against FP64 at
-    the edges of the 64x16 tiles.  A fraction's error: the powers' 1e-7 (p 4.5:
+    the edges of the tiles.  A fraction's error: the powers' 1e-7 (p 4.5:
     the slope's rounding times p) twice, and its own rounding."""
     from paper_2606_12800_gb300 import api
     z = inputs.fractal_dem(*shape, beta=2.0, tilt=0.0, seed=6)
