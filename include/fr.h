@@ -88,16 +88,18 @@ typedef enum {
  *                  check synchronises the stream).
  * Global phase of D8 accumulation (fr_accumulate with a D8 routing, whose
  * fr_routing.flags carry these, and fr_route_d8).  Cells whose upstream basin
- * leaves their tile are finished either by walkers that follow the receivers
- * one cell per step, or by a solve on the skeleton of a 64x64 tiling whose
- * steps cross a whole tile (Sec. 2.4's skeleton of the domain decomposition);
- * the second wins on DEMs with long rivers (depression-filled, planar), the
- * first on rough ones.  By default the library picks the skeleton solve when
- * at least 1/512 of the cells need the global phase.  Both give the same
- * areas; real-valued water differs only in the order of two-float additions.
- *   FR_GLOBAL_WALKERS  always the cell walkers.
+ * leaves their tile are finished either cell by cell along the receivers (the
+ * cell walkers; while they are few, threads that own some of them and read
+ * their donors until those are there), or by a solve on the skeleton of a
+ * tiling (64x64 for areas, 32x32 with water) whose steps cross a whole tile
+ * (Sec. 2.4's skeleton of the domain decomposition); the second wins on DEMs
+ * with long rivers (depression-filled, planar), the first on rough ones.  By
+ * default the library picks the skeleton solve when at least 1/512 of the
+ * cells need the global phase.  Both give the same areas; real-valued water
+ * differs only in the order of two-float additions.
+ *   FR_GLOBAL_WALKERS  always cell by cell.
  *   FR_GLOBAL_SKELETON always the skeleton solve (grids too small for its
- *                  scratch, under about 64x64 cells, use the walkers).
+ *                  scratch, under about 64x64 cells, go cell by cell).
  * Routing flag of MFD routings (fr_routing.flags), for fr_accumulate and
  * fr_route_adjoint: the checkpoint of the weights between a forward route and
  * its adjoint.  By default both calls recompute the fractions from the DEM
@@ -431,8 +433,9 @@ fr_status fr_receiver_index(const uint8_t* dir, int64_t nx, int64_t ny, int32_t 
                             void* idx_out, void* stream);
 
 /*
- * Time limit of device-side waits (the grid barrier between the rounds of the
- * MFD and adjoint global phases), in nanoseconds of the GPU's global timer; a
+ * Time limit of device-side waits (in the MFD and adjoint global phases, the
+ * time without progress and the grid barrier between rounds; in the tiled D8
+ * receivers, a copy's arrival), in nanoseconds of the GPU's global timer; a
  * wait that runs out leaves FR_ERR_NO_PROGRESS in the status word and the
  * kernel returns.  Applies to calls enqueued after it, in every thread of the
  * process.  Default 10 s.  Returns the previous limit.

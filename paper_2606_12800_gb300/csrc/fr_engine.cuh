@@ -14,15 +14,17 @@
 //     region are marked "global" (a bit per cell and a list).
 //  2. global phase (this file, a second kernel): instead of the paper's
 //     Richardson iteration across subdomain boundaries (App. B.1) the global
-//     cells are solved exactly.  Each global cell has an arrival counter for
-//     its global dependencies.  For D8 forward routing (one receiver per cell)
-//     a cell with none starts a walker, each finished cell increments its
+//     cells are solved exactly.  When there are few, every lane of a
+//     cooperative kernel owns some and reads their dependencies until they are
+//     there (k_global_poll).  More than that go by arrival counters, one per
+//     global cell.  For D8 forward routing (one receiver per cell) a cell with
+//     no global dependency starts a walker, each finished cell increments its
 //     receiver's counter, and the thread that completes a counter computes
-//     that cell ("last arriver continues"); no thread ever waits on another.
-//     For the modes where one cell can make several cells ready (MFD forward,
-//     both adjoints) the global cells are processed in rounds instead (see
-//     k_global_levels).  A routing graph with a cycle cannot hang either
-//     kernel: its cells are never reached, which the completion count reports.
+//     that cell ("last arriver continues"); no thread waits on another.  For
+//     the modes where one cell can make several cells ready (MFD forward, both
+//     adjoints) they are processed in rounds (see k_global_levels).  A routing
+//     graph with a cycle cannot hang any of these: its cells are never
+//     reached, which the completion count reports.
 //
 // Values are pulled from dependencies in a fixed order, so results are
 // bit-reproducible.  Real-valued sums are two-float (fp32 hi + lo); unit-rain
@@ -606,8 +608,8 @@ __global__ void __launch_bounds__(256) k_global_levels(const Prob* __restrict__ 
 //
 // A lane tries its cells in turn and never waits at one, and the launch is
 // cooperative (every lane runs), so an acyclic routing always gets on.  Where
-// nothing has been finished anywhere for kPollStuck tries (a cycle), or for the
-// wait limit, the lanes leave; the completion count reports the rest.
+// nothing has been finished anywhere for kPollStuck tries (a cycle), or (MFD and
+// the adjoints) for the wait limit, the lanes leave; the completion count reports the rest.
 constexpr int kPollCells = 4;
 constexpr int kPollStuck = 1 << 14;
 constexpr uint32_t kPending = 0xFFC0DEADu;
@@ -822,7 +824,8 @@ cudaError_t launch_global(const Prob* probs, const Prob& single, EngineGlobals* 
     const Prob* pp = probs;
     unsigned long long total = total_cells;
     unsigned long long poll_max = (unsigned long long)gp * 256 * kPollCells;
-    unsigned long long limit = wait_limit_ns();
+    // D8 forward: no wait limit, as the walkers have none (a cycle ends at kPollStuck)
+    unsigned long long limit = M == Mode::FwdD8 ? ~0ull : wait_limit_ns();
     void* args[] = {(void*)&pp, (void*)&one, (void*)&G, (void*)&total, (void*)&poll_max, (void*)&limit};
     // no more blocks than the grid could fill with global cells
     const unsigned long long most = (total_cells + 255) / 256;

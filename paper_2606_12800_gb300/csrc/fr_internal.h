@@ -34,7 +34,7 @@ struct Prob {
     float* out_lo;         // value trailing word (user output or workspace)
     uint64_t* area;        // D8 forward unit-rain areas or NULL
     uint32_t* cnt;         // packed byte arrival counters, zeroed before the launch
-    int64_t* link;         // 8 B/cell scratch: frontier buffer of the global rounds
+    int64_t* link;         // 8 B/cell scratch: walkers' start list (D8), frontier buffer of the rounds
     uint32_t* gbits;       // one bit per cell: "global" (solved by the walkers), zeroed
     unsigned long long* glist;  // compact list of global cells (pid << 40 | cell)
     int64_t glist_cap;     // capacity of glist (entries)
@@ -62,8 +62,8 @@ struct EngineGlobals {
     unsigned long long fcount[3];    // level-synchronous global phase: frontier sizes
     unsigned int bar_count;          // grid barrier: blocks arrived
     unsigned int bar_gen;            // grid barrier: generation
-    unsigned long long rounds;       // level-synchronous global phase: rounds run (diagnostic)
-    unsigned long long unused;
+    unsigned long long rounds;       // polling: cells finished so far; level-synchronous phase: rounds run
+    unsigned long long unused;       // keeps the words behind it in place
     unsigned long long sink_area;    // D8 areas: sum of the areas of the FR_SINK cells the local phase finished
     unsigned long long pad[2];
 };

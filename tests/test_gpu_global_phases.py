@@ -50,3 +50,20 @@ def test_plane_walked(shape):
     ref = np.broadcast_to(np.arange(1, nx + 1), (ny, nx))
     np.testing.assert_array_equal(o["area"].cpu().numpy(), ref)
     np.testing.assert_array_equal(o["w"].cpu().numpy(), ref.astype(np.float32))
+
+
+def test_d8_polling_has_no_wait_limit():
+    """The wait limit is for the MFD and adjoint phases: a D8 accumulation whose
+    global cells are polled finishes under a limit of zero, as the walkers do."""
+    from paper_2606_12800_gb300 import api
+    z = inputs.fractal_dem(300, 700, beta=2.1, tilt=0.0, seed=22)
+    d, _, _, order = oracle.route_d8(z, 30.0)
+    _, a = oracle.accumulate_d8(d, order, None)
+    R = api.routing_d8(torch.from_numpy(d).cuda(), WALK)
+    prev = api.set_wait_limit(0)
+    try:
+        o = api.accumulate(R, None, want_w=False, want_area=True, device="cuda")
+        assert api.get_status() == 0
+    finally:
+        api.set_wait_limit(prev)
+    np.testing.assert_array_equal(o["area"].cpu().numpy().astype(np.uint64), a)
