@@ -833,10 +833,11 @@ cudaError_t launch_global(const Prob* probs, const Prob& single, EngineGlobals* 
     e = cudaLaunchCooperativeKernel((const void*)k_global_poll<M, W, AREA>, dim3(blocks), dim3(256), args, 0, s);
     if (e != cudaSuccess || total_cells <= poll_max) return e;
     if constexpr (M == Mode::FwdD8) {
-        k_global_init<M, W, AREA><<<walker_grid() / 2, 256, 0, s>>>(probs, single, G, poll_max);
+        const unsigned wb = walker_blocks(total_cells);
+        k_global_init<M, W, AREA><<<wb, 256, 0, s>>>(probs, single, G, poll_max);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        k_global<M, W, AREA><<<walker_grid() / 2, 256, 0, s>>>(probs, single, G, total_cells, poll_max);
+        k_global<M, W, AREA><<<wb, 256, 0, s>>>(probs, single, G, total_cells, poll_max);
         return cudaGetLastError();
     } else {
         static int grid_lev[64] = {};

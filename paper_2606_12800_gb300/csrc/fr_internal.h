@@ -73,6 +73,16 @@ enum class Mode : int { FwdD8 = 0, FwdMfd = 1, AdjD8 = 2, AdjMfd = 3 };
 
 // Grid of the D8 forward walker kernel (fr_accumulate.cu).
 int walker_grid();
+// Blocks of the walker kernels on n cells: half the grid up to 2^24 cells, where
+// an idle launch is the usual case and the walkers gain nothing from more (filled
+// 4096^2 19.1 ms either way); all of it above 2^25, where a thread that follows a
+// trunk keeps its other starts waiting (filled 32768^2, forced walkers, half the
+// grid 1043 ms, all of it 370 to 615 from call to call).
+inline unsigned walker_blocks(unsigned long long n) {
+    const unsigned all = (unsigned)walker_grid(), half = all / 2;
+    const unsigned long long want = n >> 15;
+    return want < half ? half : want < all ? (unsigned)want : all;
+}
 // Time a device-side wait may take before the call reports
 // FR_ERR_NO_PROGRESS (fr_set_wait_limit; fr_api.cu).
 unsigned long long wait_limit_ns();
