@@ -67,3 +67,24 @@ def test_d8_polling_has_no_wait_limit():
     finally:
         api.set_wait_limit(prev)
     np.testing.assert_array_equal(o["area"].cpu().numpy().astype(np.uint64), a)
+
+
+@pytest.mark.parametrize("shape", [(300, 517), (4100, 4163)])
+def test_skeleton_looks_ahead(shape):
+    """The skeleton forced on rough terrain, where most tiles hold no global cell
+    and a block goes through several flags' worth of tiles (rows that share
+    words of the bitmap): the walkers' areas, and their water to two roundings."""
+    from paper_2606_12800_gb300 import api
+    z = torch.from_numpy(inputs.fractal_dem(*shape, beta=2.1, tilt=0.0, seed=23)).cuda()
+    d = api.receivers_d8(z, 30.0, 0)
+    out = {}
+    for f in (SKEL, WALK):
+        for want_w in (True, False):
+            out[f, want_w] = api.accumulate(api.routing_d8(d, f), None, want_w=want_w, want_area=True,
+                                            device=d.device)
+            assert api.get_status() == 0
+    ref = out[WALK, False]["area"]
+    for k, o in out.items():
+        assert torch.equal(o["area"], ref)
+        if k[1]:
+            torch.testing.assert_close(o["w"], ref.float(), rtol=2 * 2.0 ** -23, atol=0)
