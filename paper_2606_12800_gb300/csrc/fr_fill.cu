@@ -222,11 +222,11 @@ __global__ void __launch_bounds__(kFNT) k_fill_sweep(const float* __restrict__ z
             put(r, kFR - 1, cz[1], cf[1]);
         }
     }
-    if (threadIdx.x == 0) {
-        S.flags = 0;
-        if (!FIRST) act[blockIdx.x] = 0;  // this record serves the sweep after next again
-    }
+    if (threadIdx.x == 0) S.flags = 0;
     __syncthreads();
+    // this record serves the sweep after next again; cleared behind the barrier,
+    // when every thread of the block has read it
+    if (!FIRST && threadIdx.x == 0) act[blockIdx.x] = 0;
     // the boundary's values as loaded
     constexpr int NB = 4 * kFT - 4;
     constexpr int NQB = (NB + kFNT - 1) / kFNT;  // boundary cells a thread
