@@ -617,6 +617,33 @@ constexpr uint64_t kPendingArea = ~0ull;  // areas: above any count of cells
 
 __device__ __forceinline__ bool pending(float v) { return __float_as_uint(v) == kPending; }
 
+// What one lane stores while another reads it: relaxed at device scope on both
+// sides, each word whole and seen in time.  A value needs no order beside its own
+// words, so there are no fences (and L1, which these pass by, was never used).
+__device__ __forceinline__ float poll_ld(const float* a, const Prob& P, int64_t i, unsigned site) {
+    float v = 0.0f;
+    if (FR_OK(i, ncell(P), site)) asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(v) : "l"(a + i));
+    return v;
+}
+__device__ __forceinline__ void poll_st(float* a, const Prob& P, int64_t i, float v, unsigned site) {
+    if (FR_OK(i, ncell(P), site)) asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" ::"l"(a + i), "f"(v) : "memory");
+}
+__device__ __forceinline__ df poll_value(const Prob& P, int64_t i) {
+    return {poll_ld(P.out_hi, P, i, 11), poll_ld(P.out_lo, P, i, 12)};
+}
+__device__ __forceinline__ void poll_put(const Prob& P, int64_t i, df v) {
+    poll_st(P.out_hi, P, i, v.hi, 13);
+    poll_st(P.out_lo, P, i, v.lo, 14);
+}
+__device__ __forceinline__ uint64_t poll_area(const Prob& P, int64_t i) {
+    uint64_t v = 0;
+    if (FR_OK(i, ncell(P), 3)) asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(P.area + i));
+    return v;
+}
+__device__ __forceinline__ void poll_put_area(const Prob& P, int64_t i, uint64_t v) {
+    if (FR_OK(i, ncell(P), 4)) asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(P.area + i), "l"(v) : "memory");
+}
+
 // Row and column of cell t (32-bit division where the grid allows it).
 __device__ __forceinline__ void cell_xy(const Prob& P, int64_t t, int64_t& x, int64_t& y) {
     y = ((uint64_t)ncell(P) >> 32) ? t / P.nx : (int64_t)((uint32_t)t / (uint32_t)P.nx);
@@ -644,10 +671,10 @@ __device__ __forceinline__ bool poll_step_d8(const Prob& P, int64_t t) {
         vv[k] = df_make(0.0f);
         a[k] = 0;
         if constexpr (E::kVal) {
-            if (on) vv[k] = g_value<E>(P, j);
+            if (on) vv[k] = poll_value(P, j);
         }
         if constexpr (E::kArea) {
-            if (on) a[k] = rd_area(P, j);
+            if (on) a[k] = poll_area(P, j);
         }
     }
 #pragma unroll
@@ -658,14 +685,13 @@ __device__ __forceinline__ bool poll_step_d8(const Prob& P, int64_t t) {
 #pragma unroll
         for (int k = 0; k < 8; ++k)
             if ((don >> k) & 1u) v = df_add(v, vv[k]);
-        wr_f(P.out_hi, P, t, v.hi, 13);
-        wr_f(P.out_lo, P, t, v.lo, 14);
+        poll_put(P, t, v);
     }
     if constexpr (E::kArea) {
         uint64_t s = 1;
 #pragma unroll
         for (int k = 0; k < 8; ++k) s += a[k];
-        wr_area(P, t, s);
+        poll_put_area(P, t, s);
     }
     return true;
 }
@@ -696,7 +722,7 @@ __device__ __forceinline__ bool poll_step(const Prob& P, int64_t t) {
         vv[k] = df_make(0.0f);
         if (!((dep >> k) & 1u)) continue;
         const int64_t j = t + offi(k, P.nx);
-        vv[k] = g_value<E>(P, j);
+        vv[k] = poll_value(P, j);
         f[k] = 1.0f;
         if constexpr (E::kMfd) f[k] = E::kAdj ? __ldg(P.frac + t * 8 + k) : __ldg(P.frac + j * 8 + opp(k));
     }
@@ -704,8 +730,7 @@ __device__ __forceinline__ bool poll_step(const Prob& P, int64_t t) {
     for (int k = 0; k < 8; ++k) ready &= !pending(vv[k].hi) && !pending(vv[k].lo);
     if (!ready) return false;
     const df v = df_dot8(init_value<E>(P, t, recv), f, vv);  // the fixed order
-    wr_f(P.out_hi, P, t, v.hi, 13);
-    wr_f(P.out_lo, P, t, v.lo, 14);
+    poll_put(P, t, v);
     return true;
 }
 
