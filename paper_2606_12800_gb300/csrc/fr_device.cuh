@@ -122,12 +122,17 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));  // of NaN and a number, the number
     return r;
 }
+__device__ __forceinline__ float min3(float a, float b, float c) {
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
 
 // The same selection for the rule fixed at compile time: the largest of the
 // eight keys s_k by three-input maxima, then the first code that has it (a NaN
-// key equals nothing).  A positive largest key belongs to a lower neighbour and
-// a negative one to none; a zero or NaN one (returned in m) leaves the choice to
-// d8_code: the neighbours are level, or a drop has underflowed.
+// key equals nothing).  A positive largest key belongs to a lower neighbour; a
+// negative one, or NaN in all eight, to none.  Zero (returned in m) is level
+// ground, or a drop whose product has underflowed: see d8_unsure.
 template <bool LOWEST>
 __device__ __forceinline__ uint32_t d8_code_max(float zc, const float (&zn)[8], float c_orth,
                                                 float c_diag, float& m) {
@@ -143,10 +148,24 @@ __device__ __forceinline__ uint32_t d8_code_max(float zc, const float (&zn)[8], 
     for (int k = 6; k >= 0; --k) code = s[k] == m ? (uint32_t)k : code;
     return m > 0.0f ? code : kSink;
 }
-// Whether one of four largest keys is zero or NaN (or so small that their
-// product underflows): their cells are chosen again by d8_code.
-__device__ __forceinline__ bool d8_unsure(const float (&m)[4]) {
-    return !(fabsf(__fmul_rn(__fmul_rn(m[0], m[1]), __fmul_rn(m[2], m[3]))) > 0.0f);
+// Whether the codes of four cells with largest keys m have to come from d8_code:
+// a key is zero although a neighbour is lower.  lower(q) says whether cell q has
+// a lower neighbour; it is asked only where a product of the keys is zero or NaN.
+// Differences of floats do not underflow, so the lowest-neighbour rule never has to.
+// Level ground is ordinary (whole metres, lakes, no-data areas): 16384^2, rough /
+// whole metres / a lake / all level 490 / 527 / 531 / 580 us; 511 / 875 / 883 / 1350
+// with d8_code for every zero key, 613 on all four with a running best over the directions.
+template <bool LOWEST, class F>
+__device__ __forceinline__ bool d8_unsure(const float (&m)[4], F lower) {
+    if (LOWEST || fabsf(__fmul_rn(__fmul_rn(m[0], m[1]), __fmul_rn(m[2], m[3]))) > 0.0f) return false;
+    bool hidden = false;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) hidden |= (m[q] == 0.0f) & lower(q);
+    return hidden;
+}
+// Whether one of the eight elevations is below zc.
+__device__ __forceinline__ bool d8_any_lower(float zc, const float (&zn)[8]) {
+    return min3(min3(zn[0], zn[1], zn[2]), min3(zn[3], zn[4], zn[5]), fminf(zn[6], zn[7])) < zc;
 }
 
 // ------------------------------------------------------------ MFD weights

@@ -107,13 +107,19 @@ __device__ __forceinline__ void recv_d8_strip_t(const float* __restrict__ z, int
         spread(rows[r + 2], c);
         uint32_t codes[4];
         float m[4];
+        struct Around {
+            float z[8];
+        };
+        auto around = [&](int g) -> Around {
+            return {{b.r[g], a.c[g], b.l[g], c.c[g], D4 ? inf : a.r[g], D4 ? inf : a.l[g], D4 ? inf : c.l[g],
+                     D4 ? inf : c.r[g]}};
+        };
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
-            const float zn[8] = {b.r[g], a.c[g], b.l[g], c.c[g], D4 ? inf : a.r[g], D4 ? inf : a.l[g],
-                                 D4 ? inf : c.l[g], D4 ? inf : c.r[g]};
-            codes[g] = d8_code_max<LOWEST>(b.c[g], zn, c_orth, c_diag, m[g]);
+            codes[g] = d8_code_max<LOWEST>(b.c[g], around(g).z, c_orth, c_diag, m[g]);
+            if (!INTERIOR && x0 + lane + 32 * g >= nx) m[g] = 1.0f;  // off the grid: no key
         }
-        if (d8_unsure(m)) {
+        if (d8_unsure<LOWEST>(m, [&](int g) { return d8_any_lower(b.c[g], around(g).z); })) {
 #pragma unroll 1
             for (int g = 0; g < 4; ++g) {
                 const int64_t gx = x0 + lane + 32 * g;
@@ -301,8 +307,8 @@ __global__ void __launch_bounds__(256) k_receivers_d8_tma(const __grid_constant_
         // and tile origin are multiples of four (the tensor map's condition), so
         // a group of four cells lies in the grid or outside it.
         uint8_t* const out = dir + y0 * nx + x0 + qx;
-        const bool cols = x0 + qx < nx;
-        for (int r = 2 * warp; r < TTY; r += 16) {
+        const int rows = x0 + qx < nx ? (int)(ny - y0 < TTY ? ny - y0 : TTY) : 0;  // none for a lane off the grid
+        for (int r = 2 * warp; r < rows; r += 16) {
             // buffer rows r .. r + 3, columns qx + 3 .. qx + 8 (tile column c
             // sits at buffer column c + 4)
             float w[4][6];
@@ -321,16 +327,19 @@ __global__ void __launch_bounds__(256) k_receivers_d8_tma(const __grid_constant_
             for (int h = 0; h < 2; ++h) {
                 uint32_t codes[4];
                 float m[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
+                struct Around {
+                    float z[8];
+                };
+                auto around = [&](int q) -> Around {
                     const int c = q + 1;  // window column of the cell
                     const float inf = __int_as_float(0x7f800000);
-                    const float zn[8] = {w[h + 1][c + 1], w[h][c], w[h + 1][c - 1], w[h + 2][c],
-                                         D4 ? inf : w[h][c + 1], D4 ? inf : w[h][c - 1],
-                                         D4 ? inf : w[h + 2][c - 1], D4 ? inf : w[h + 2][c + 1]};
-                    codes[q] = d8_code_max<LOWEST>(w[h + 1][c], zn, c_orth, c_diag, m[q]);
-                }
-                if (d8_unsure(m)) {
+                    return {{w[h + 1][c + 1], w[h][c], w[h + 1][c - 1], w[h + 2][c], D4 ? inf : w[h][c + 1],
+                             D4 ? inf : w[h][c - 1], D4 ? inf : w[h + 2][c - 1], D4 ? inf : w[h + 2][c + 1]}};
+                };
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    codes[q] = d8_code_max<LOWEST>(w[h + 1][q + 1], around(q).z, c_orth, c_diag, m[q]);
+                if (d8_unsure<LOWEST>(m, [&](int q) { return d8_any_lower(w[h + 1][q + 1], around(q).z); })) {
 #pragma unroll 1
                     for (int q = 0; q < 4; ++q) {
                         const float* c = b + (r + h + 1) * TBX + qx + 4 + q;
@@ -346,7 +355,7 @@ __global__ void __launch_bounds__(256) k_receivers_d8_tma(const __grid_constant_
                     }
                 }
                 if (!interior) {
-                    if (!cols || y0 + r + h >= ny) continue;
+                    if (r + h >= rows) continue;
 #pragma unroll
                     for (int q = 0; q < 4; ++q)
                         if (!edge_route && is_edge(x0 + qx + q, y0 + r + h, nx, ny)) codes[q] = kSink;
