@@ -507,7 +507,7 @@ __global__ void __launch_bounds__(Gm::NT, d8_blocks<Gm, W>()) k_local_d8(Prob Po
         }
         ++done;
         if constexpr (W) {
-            wr_f(P.out_hi, P, gi, S.vhi[r], 27);
+            wr_f(P.out_hi, P, gi, final_word(S.vhi[r]), 27);
             if (P.lo_full || need_lo_of(r, lx, ly)) wr_f(P.out_lo, P, gi, S.vlo[r], 28);
         }
         if constexpr (AREA) wr_area(P, gi, 1u + (pkc & kPkArea));
@@ -526,7 +526,8 @@ __global__ void __launch_bounds__(Gm::NT, d8_blocks<Gm, W>()) k_local_d8(Prob Po
             }
             const int64_t gi = (y0 + ly) * P.nx + x0 + lx;
             if constexpr (W) {
-                const float4 v = *reinterpret_cast<const float4*>(S.vhi + r);
+                const float4 h = *reinterpret_cast<const float4*>(S.vhi + r);
+                const float4 v = make_float4(final_word(h.x), final_word(h.y), final_word(h.z), final_word(h.w));
                 if (vec) {
                     *reinterpret_cast<float4*>(P.out_hi + gi) = v;
                 } else {

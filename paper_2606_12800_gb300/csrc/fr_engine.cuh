@@ -616,6 +616,10 @@ constexpr uint32_t kPending = 0xFFC0DEADu;
 constexpr uint64_t kPendingArea = ~0ull;  // areas: above any count of cells
 
 __device__ __forceinline__ bool pending(float v) { return __float_as_uint(v) == kPending; }
+// The leading word of a final cell as the local phases publish it.  A cell that
+// got nothing holds the caller's rain untouched, which may be a NaN of any
+// pattern, the pending one too: it becomes the NaN that sums yield.
+__device__ __forceinline__ float final_word(float v) { return pending(v) ? __int_as_float(0x7fffffff) : v; }
 
 // What one lane stores while another reads it: relaxed at device scope on both
 // sides, each word whole and seen in time.  A value needs no order beside its own

@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(kHaloNT, 1) k_local_halo(Prob Pone, EngineGlob
             if (!fin1) continue;
             ++done;
             const float2 a = S.v[ey * EX + ex];
-            wr_f(P.out_hi, P, gi, a.x, 27);
+            wr_f(P.out_hi, P, gi, final_word(a.x), 27);
             wr_f(P.out_lo, P, gi, a.y, 28);
         }
     }
