@@ -30,6 +30,11 @@
  *           stream).  All work is enqueued on it; calls return without
  *           synchronising.  Inputs must stay valid and outputs must not be
  *           read until the stream has reached the end of the call.
+ *           The slope-split and adjoint calls launch cooperative kernels that
+ *           fill the device: on a stream that may use only some of its SMs (a
+ *           green context, a share of MPS) they return FR_ERR_CUDA, and a graph
+ *           captured from them must not be launched on such a stream, where it
+ *           would not start.  D8 calls run there, and captured ones too.
  * Errors    argument errors are detected synchronously and returned before
  *           anything is enqueued.  Launch errors return FR_ERR_CUDA.  Errors
  *           found on the device (a routing graph with a cycle, a device-side

@@ -859,9 +859,28 @@ cudaError_t launch_global(const Prob* probs, const Prob& single, EngineGlobals* 
     // no more blocks than the grid could fill with global cells
     const unsigned long long most = (total_cells + 255) / 256;
     const unsigned blocks = most < (unsigned long long)gp ? (unsigned)(most ? most : 1) : (unsigned)gp;
-    e = cudaLaunchCooperativeKernel((const void*)k_global_poll<M, W, AREA>, dim3(blocks), dim3(256), args, 0, s);
-    if (e != cudaSuccess || total_cells <= poll_max) return e;
     if constexpr (M == Mode::FwdD8) {
+        // Polling needs every lane to run, so it is a cooperative launch that fills
+        // the device.  A stream that may use only some of the SMs (a green context,
+        // a share of MPS) refuses that; a graph would take it, wherever it is launched
+        // later, and never start it.  There the walkers, which wait for no other block,
+        // take all cells.
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+            (void)cudaGetLastError();
+            cap = cudaStreamCaptureStatusNone;
+        }
+        if (cap == cudaStreamCaptureStatusNone) {
+            e = cudaLaunchCooperativeKernel((const void*)k_global_poll<M, W, AREA>, dim3(blocks), dim3(256), args, 0, s);
+            if (e != cudaErrorCooperativeLaunchTooLarge) {
+                if (e != cudaSuccess || total_cells <= poll_max) return e;
+            } else {
+                (void)cudaGetLastError();
+                poll_max = 0;
+            }
+        } else {
+            poll_max = 0;
+        }
         const unsigned wb = walker_blocks(total_cells);
         k_global_init<M, W, AREA><<<wb, 256, 0, s>>>(probs, single, G, poll_max);
         e = cudaGetLastError();
@@ -869,6 +888,8 @@ cudaError_t launch_global(const Prob* probs, const Prob& single, EngineGlobals* 
         k_global<M, W, AREA><<<wb, 256, 0, s>>>(probs, single, G, total_cells, poll_max);
         return cudaGetLastError();
     } else {
+        e = cudaLaunchCooperativeKernel((const void*)k_global_poll<M, W, AREA>, dim3(blocks), dim3(256), args, 0, s);
+        if (e != cudaSuccess || total_cells <= poll_max) return e;
         static int grid_lev[64] = {};
         int gl = 0;
         // one block per SM: a round's frontier (about 20 K cells on an 8192^2
