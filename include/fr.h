@@ -96,7 +96,8 @@ typedef enum {
  * leaves their tile are finished either cell by cell along the receivers (the
  * cell walkers; while they are few, threads that own some of them and read
  * their donors until those are there), or by a solve on the skeleton of a
- * tiling (64x64 for areas, 32x32 with water) whose steps cross a whole tile
+ * tiling (64x64 for areas and for long, narrow grids, else 32x32 with water)
+ * whose steps cross a whole tile
  * (Sec. 2.4's skeleton of the domain decomposition); the second wins on DEMs
  * with long rivers (depression-filled, planar), the first on rough ones.  By
  * default the library picks the skeleton solve when at least 1/512 of the

@@ -128,8 +128,8 @@ bool routing_ok(const fr_routing* R) {
     return false;
 }
 
-// with_water: the D8 accumulation solves water (the skeleton's tile size).
-Prob base_prob(const fr_routing* R, char* ws, bool with_water = false) {
+// with_water, with_area: what the D8 accumulation solves (the skeleton's tile size).
+Prob base_prob(const fr_routing* R, char* ws, bool with_water = false, bool with_area = true) {
     Layout L = layout(R->nx * R->ny);
     Prob P;
     std::memset(&P, 0, sizeof(P));
@@ -148,7 +148,8 @@ Prob base_prob(const fr_routing* R, char* ws, bool with_water = false) {
     // slots
     P.skel_min = ~0ull;
     if (R->kind == FR_ROUTING_D8) {
-        const int side = skel_side(with_water);
+        const int side = skel_side(with_water, with_area, R->nx, R->ny);
+        P.skel_side = side;
         const int64_t n = R->nx * R->ny, st = skel_tiles(R->nx, R->ny, side);
         const size_t o_pool = align256((size_t)st * (4 * side - 4) * 8);
         const size_t need = o_pool + (size_t)st * skel_pool(side) * 2;
@@ -280,7 +281,7 @@ fr_status accumulate_impl(const fr_routing* R, const float* rain, float* w_out, 
     if (mfd && (area_out || !w_out)) return FR_ERR_INVALID_ARG;
     const int64_t n = R->nx * R->ny;
     if (!(mfd ? ws_ok_mfd(ws, ws_bytes, n) : ws_ok(ws, ws_bytes, n))) return FR_ERR_WORKSPACE;
-    Prob P = base_prob(R, (char*)ws, w_out != nullptr);
+    Prob P = base_prob(R, (char*)ws, w_out != nullptr, area_out != nullptr);
     P.init = rain;
     P.out_hi = w_out;
     if (w_lo_out) {

@@ -40,6 +40,7 @@ struct Prob {
     int64_t glist_cap;     // capacity of glist (entries)
     MfdConst mc;
     int32_t lo_full;       // out_lo is a user output: write it for every cell
+    int32_t skel_side;     // side of the skeleton's tiles (32 or 64)
     // D8 forward global phase: the tile-skeleton solve (fr_skel.cu) runs when
     // the local phase leaves at least skel_min global cells, the cell walkers
     // otherwise (~0: walkers always)
@@ -92,10 +93,21 @@ cudaError_t read_clear_tma_error(unsigned* out, cudaStream_t s);
 // Linear receiver index of every cell from D8 codes (fr_receivers.cu).
 cudaError_t launch_receiver_index(const uint8_t* dir, int64_t nx, int64_t ny, bool wide, void* out,
                                   cudaStream_t s);
-// Skeleton tiles of the D8 global phase (fr_skel.cu): side x side cells, with
-// water or areas alone; dependency slots per tile (a dependency is a donor in
-// the one-cell ring around the tile, and each ring cell has one receiver).
-__host__ __device__ constexpr int skel_side(bool with_water) { return with_water ? 32 : 64; }
+// Skeleton tiles of the D8 global phase (fr_skel.cu): side x side cells;
+// dependency slots per tile (a dependency is a donor in the one-cell ring around
+// the tile, and each ring cell has one receiver).
+// Side: 64 for areas alone.  With water 32 (see SkGeo), but for long, narrow
+// grids: a river along the grid crosses twice as many 32x32 tiles, one dependent
+// step each, while the tile passes that these shorten grow with the width only.
+// Measured with tiles of 32 / 64, us a call: water and areas, planes of 256x16384
+// 2542 / 2037, 512x16384 3099 / 3039, 700x16384 3468 / 3727, 256x2000 365 / 317,
+// filled 256x4000 512 / 456, 512x4000 621 / 663; water alone (of which two 64x64
+// tiles fit an SM), planes of 1024x16384 3627 / 3227, 2048x16384 5351 / 5333,
+// 1000x4000 946 / 904, filled 1500x16384 3214 / 2988, 128x2000 249 / 270.
+inline int skel_side(bool with_water, bool with_area, int64_t nx, int64_t ny) {
+    const int64_t longer = nx > ny ? nx : ny, shorter = nx > ny ? ny : nx;
+    return with_water && (longer < 2048 || shorter > (with_area ? 320 : 1536)) ? 32 : 64;
+}
 __host__ __device__ constexpr int skel_pool(int side) { return 4 * side + 4; }
 __host__ __device__ inline int64_t skel_tiles(int64_t nx, int64_t ny, int side) {
     return ((nx + side - 1) / side) * ((ny + side - 1) / side);

@@ -50,18 +50,19 @@
 namespace fr {
 namespace {
 
-// Tile sides.  Areas alone: 64 (three blocks of 256 threads per SM; 32 measured
-// the same in the tile passes, with twice the steps in between).  With water a
-// cell takes 28 bytes of shared memory, so a 64x64 tile leaves room for one
-// block per SM and its chain of latencies is exposed: 32x32 tiles, six blocks of
-// 128 threads, took passes A and C of a filled 4096^2 DEM from 922 and 773 to
-// 331 and 289 us.
-template <bool W>
+// Tile sides (chosen by skel_side).  Areas alone: 64 (three blocks of 256 threads
+// per SM; 32 measured the same in the tile passes, with twice the steps in
+// between).  With water a cell takes 28 bytes of shared memory (20 without areas),
+// so a 64x64 tile leaves room for one block per SM (two) and its chain of
+// latencies is exposed: 32x32 tiles, six blocks of 128 threads, took passes A and C
+// of a filled 4096^2 DEM from 922 and 773 to 331 and 289 us.  On long, narrow grids
+// the steps in between weigh more, and 64x64 stays.
+template <bool W, int SIDE>
 struct SkGeo {
-    static constexpr int SX = skel_side(W), SY = SX, SN = SX * SY;
+    static constexpr int SX = SIDE, SY = SX, SN = SX * SY;
     static constexpr int SRX = SX + 2, SRY = SY + 2, SRN = SRX * SRY;  // with a one-cell ring
-    static constexpr int NT = W ? 128 : 256;                           // threads of the tile passes
-    static constexpr int kBlocks = W ? 6 : 3;                          // blocks per SM asked of the compiler
+    static constexpr int NT = SIDE == 32 ? 128 : 256;                     // threads of the tile passes
+    static constexpr int kBlocks = SIDE == 32 ? 6 : 3;           // blocks per SM asked of the compiler
     static constexpr int kPool = skel_pool(SX);
     static_assert(SN <= 4096, "local indices take 12 bits");
     static_assert(kPool == 2 * (SX + SY) + 4, "dependency slots per tile: the ring cells");
@@ -106,9 +107,9 @@ struct TileGeo {
     int tiles_x;
 };
 
-template <bool W>
+template <int SIDE>
 __device__ __forceinline__ TileGeo tile_geo(const Prob& P, int64_t t) {
-    constexpr int SX = SkGeo<W>::SX, SY = SkGeo<W>::SY;
+    constexpr int SX = SIDE, SY = SIDE;
     TileGeo g;
     g.tiles_x = (int)((P.nx + SX - 1) / SX);
     const int64_t ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
@@ -147,9 +148,9 @@ __device__ __forceinline__ int bindex(int lx, int ly, int ex, int ey) {
     return ex + (ly - 1) * per + (lx == 0 ? 0 : 1);
 }
 
-template <bool W, bool AREA>
-struct SmemSk : SkGeo<W> {
-    using Geo = SkGeo<W>;
+template <bool W, bool AREA, int SIDE>
+struct SmemSk : SkGeo<W, SIDE> {
+    using Geo = SkGeo<W, SIDE>;
     static constexpr int SX = Geo::SX, SN = Geo::SN, SRN = Geo::SRN, kSkNT = Geo::NT;
     static constexpr bool kPush = AREA && !W;
     uint8_t cg[SRN];                                    // ring layout: code | kGlob
@@ -199,7 +200,7 @@ __device__ __forceinline__ void start_tiles(S_& S, unsigned long long count, int
     __syncthreads();
 }
 
-template <bool W, class S_>
+template <class S_>
 __device__ __forceinline__ int64_t next_tile(S_& S, const Prob& P, int64_t ntiles, int& step) {
     constexpr int NW = S_::kSkNT / 32;
     for (;;) {
@@ -210,7 +211,7 @@ __device__ __forceinline__ int64_t next_tile(S_& S, const Prob& P, int64_t ntile
             const int64_t tw = t + (int64_t)warp * gridDim.x;
             uint32_t any = 0;
             if (tw < ntiles) {
-                const TileGeo g = tile_geo<W>(P, tw);
+                const TileGeo g = tile_geo<S_::SX>(P, tw);
                 for (int ly = lane; ly < g.ey; ly += 32) {
                     const int64_t b0 = (g.y0 + ly) * P.nx + g.x0, b1 = b0 + g.ex - 1;  // first and last bit
                     for (int64_t w = b0 >> 5; w <= b1 >> 5; ++w) {
@@ -636,10 +637,10 @@ __device__ void walk_pull(S_& S) {
 }
 
 // Pass A: in-tile partial values, exits, entries and dependency lists.
-template <bool W, bool AREA>
-__global__ void __launch_bounds__(SkGeo<W>::NT, SkGeo<W>::kBlocks) k_skel_a(Prob P, EngineGlobals* G,
+template <bool W, bool AREA, int SIDE>
+__global__ void __launch_bounds__(SkGeo<W, SIDE>::NT, SkGeo<W, SIDE>::kBlocks) k_skel_a(Prob P, EngineGlobals* G,
                                                                             int64_t ntiles) {
-    using Sm = SmemSk<W, AREA>;
+    using Sm = SmemSk<W, AREA, SIDE>;
     constexpr int SX = Sm::SX, SRX = Sm::SRX, kSkNT = Sm::kSkNT, kSkelPool = Sm::kPool;
     constexpr bool kPush = Sm::kPush;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -648,8 +649,8 @@ __global__ void __launch_bounds__(SkGeo<W>::NT, SkGeo<W>::kBlocks) k_skel_a(Prob
     const int tid = threadIdx.x;
     int step = 0;
     start_tiles(S, __ldcg(&G->glist_count), ntiles);
-    for (int64_t t; (t = next_tile<W>(S, P, ntiles, step)) >= 0;) {
-        const TileGeo g = tile_geo<W>(P, t);
+    for (int64_t t; (t = next_tile(S, P, ntiles, step)) >= 0;) {
+        const TileGeo g = tile_geo<SIDE>(P, t);
         __syncthreads();  // the previous tile's shared memory is no longer read
         if (tid == 0) {
             S.qtail = 0;
@@ -905,10 +906,10 @@ __device__ __forceinline__ int64_t next_exit(const Prob& P, int64_t x, uint32_t 
 // their slots and values loaded eight at a time.
 // Filled 8192^2, areas 514 -> 351 us; filled 4096^2, water and areas in 32x32 tiles
 // 956 -> 624 us.
-template <bool W, bool AREA>
+template <bool W, bool AREA, int SIDE>
 __global__ void __launch_bounds__(256) k_skel_walk(Prob P, EngineGlobals* G) {
     if (__ldcg(&G->glist_count) < P.skel_min) return;
-    using Geo = SkGeo<W>;
+    using Geo = SkGeo<W, SIDE>;
     constexpr int SX = Geo::SX, SY = Geo::SY, SRX = Geo::SRX;
     const unsigned long long count = __ldcg(&G->fcount[0]);
     const int tiles_x = (int)((P.nx + SX - 1) / SX);
@@ -1016,11 +1017,11 @@ __global__ void __launch_bounds__(256) k_skel_walk(Prob P, EngineGlobals* G) {
 
 // Pass C: inflows of the entries passed down the in-tile receivers; final
 // values of the global cells; completion count.
-template <bool W, bool AREA>
-__global__ void __launch_bounds__(SkGeo<W>::NT, SkGeo<W>::kBlocks) k_skel_fix(Prob P, EngineGlobals* G,
+template <bool W, bool AREA, int SIDE>
+__global__ void __launch_bounds__(SkGeo<W, SIDE>::NT, SkGeo<W, SIDE>::kBlocks) k_skel_fix(Prob P, EngineGlobals* G,
                                                                               int64_t ntiles,
                                                                               unsigned long long total_cells) {
-    using Sm = SmemSk<W, AREA>;
+    using Sm = SmemSk<W, AREA, SIDE>;
     constexpr int SX = Sm::SX, SRX = Sm::SRX, kSkNT = Sm::kSkNT;
     constexpr bool kPush = Sm::kPush;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1031,8 +1032,8 @@ __global__ void __launch_bounds__(SkGeo<W>::NT, SkGeo<W>::kBlocks) k_skel_fix(Pr
     unsigned long long done = 0;
     int step = 0;
     start_tiles(S, __ldcg(&G->glist_count), ntiles);
-    for (int64_t t; (t = next_tile<W>(S, P, ntiles, step)) >= 0;) {
-        const TileGeo g = tile_geo<W>(P, t);
+    for (int64_t t; (t = next_tile(S, P, ntiles, step)) >= 0;) {
+        const TileGeo g = tile_geo<SIDE>(P, t);
         __syncthreads();
         if (tid == 0) {
             S.qtail = 0;
@@ -1232,29 +1233,29 @@ int persistent_grid(K kernel, int threads, size_t smem) {
     return sms * (per > 0 ? per : 1);
 }
 
-template <bool W, bool AREA>
+template <bool W, bool AREA, int SIDE>
 cudaError_t launch_skel_t(const Prob& P, EngineGlobals* G, cudaStream_t s) {
-    constexpr size_t sm = sizeof(SmemSk<W, AREA>);
+    constexpr size_t sm = sizeof(SmemSk<W, AREA, SIDE>);
     static std::atomic<unsigned long long> set_a{0}, set_c{0};
     static int grid_a = 0, grid_c = 0;
-    cudaError_t e = smem_limit_once(k_skel_a<W, AREA>, sm, set_a);
+    cudaError_t e = smem_limit_once(k_skel_a<W, AREA, SIDE>, sm, set_a);
     if (e != cudaSuccess) return e;
-    e = smem_limit_once(k_skel_fix<W, AREA>, sm, set_c);
+    e = smem_limit_once(k_skel_fix<W, AREA, SIDE>, sm, set_c);
     if (e != cudaSuccess) return e;
-    if (!grid_a) grid_a = persistent_grid(k_skel_a<W, AREA>, SkGeo<W>::NT, sm);
-    if (!grid_c) grid_c = persistent_grid(k_skel_fix<W, AREA>, SkGeo<W>::NT, sm);
+    if (!grid_a) grid_a = persistent_grid(k_skel_a<W, AREA, SIDE>, SkGeo<W, SIDE>::NT, sm);
+    if (!grid_c) grid_c = persistent_grid(k_skel_fix<W, AREA, SIDE>, SkGeo<W, SIDE>::NT, sm);
     if (!grid_a || !grid_c) return cudaErrorInvalidConfiguration;
-    const int64_t ntiles = skel_tiles(P.nx, P.ny, skel_side(W));
-    constexpr int kSkNT = SkGeo<W>::NT;
+    const int64_t ntiles = skel_tiles(P.nx, P.ny, SIDE);
+    constexpr int kSkNT = SkGeo<W, SIDE>::NT;
     const unsigned ga = (unsigned)(ntiles < grid_a ? ntiles : grid_a), gc = (unsigned)(ntiles < grid_c ? ntiles : grid_c);
-    k_skel_a<W, AREA><<<ga, kSkNT, sm, s>>>(P, G, ntiles);
+    k_skel_a<W, AREA, SIDE><<<ga, kSkNT, sm, s>>>(P, G, ntiles);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int64_t wg = (P.nx * P.ny + 255) / 256, wb = walker_blocks((unsigned long long)(P.nx * P.ny));
-    k_skel_walk<W, AREA><<<(unsigned)(wg < wb ? wg : wb), 256, 0, s>>>(P, G);
+    k_skel_walk<W, AREA, SIDE><<<(unsigned)(wg < wb ? wg : wb), 256, 0, s>>>(P, G);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_skel_fix<W, AREA><<<gc, kSkNT, sm, s>>>(P, G, ntiles, (unsigned long long)(P.nx * P.ny));
+    k_skel_fix<W, AREA, SIDE><<<gc, kSkNT, sm, s>>>(P, G, ntiles, (unsigned long long)(P.nx * P.ny));
     return cudaGetLastError();
 }
 
@@ -1262,9 +1263,10 @@ cudaError_t launch_skel_t(const Prob& P, EngineGlobals* G, cudaStream_t s) {
 
 cudaError_t launch_d8_skeleton(bool want_w, bool want_area, const Prob& P, EngineGlobals* G,
                                cudaStream_t s) {
-    if (want_w && want_area) return launch_skel_t<true, true>(P, G, s);
-    if (want_w) return launch_skel_t<true, false>(P, G, s);
-    return launch_skel_t<false, true>(P, G, s);
+    const bool wide = P.skel_side == 64;
+    if (want_w && want_area) return wide ? launch_skel_t<true, true, 64>(P, G, s) : launch_skel_t<true, true, 32>(P, G, s);
+    if (want_w) return wide ? launch_skel_t<true, false, 64>(P, G, s) : launch_skel_t<true, false, 32>(P, G, s);
+    return launch_skel_t<false, true, 64>(P, G, s);
 }
 
 }  // namespace fr
