@@ -255,13 +255,16 @@ fr_status fr_accumulate(const fr_routing* routing, const float* rain, float* w_o
  *   flags        0 or FR_CHECK_FINITE.
  *   filled_out   [ny*nx] float32, not overlapping dem.
  *   max_sweeps   >= 1: relaxation sweeps over 64x64 tiles allowed; a sweep
- *                that changes nothing ends the call (from 4096 on a mere
- *                backstop: short sweeps are run, eight of them counting as one).  FR_ERR_NO_PROGRESS if
+ *                that changes nothing ends the call.  FR_ERR_NO_PROGRESS if
  *                the surface is still moving after max_sweeps (filled_out
- *                then holds an upper bound of F).
- *   sweeps_out   host int32 or NULL: sweeps run, the last one changing nothing.
+ *                then holds an upper bound of F).  A sweep is run as up to
+ *                eight short ones; a surface that these leave moving gets
+ *                max_sweeps further sweeps in which every tile runs until it
+ *                rests.
+ *   sweeps_out   host int32 or NULL: sweeps run, the last one changing nothing;
+ *                max_sweeps where the further ones were needed.
  * Workspace: fr_workspace_size(FR_OP_FILL, nx, ny, flags).
- * Synchronises the stream after every batch of eight sweeps.
+ * Synchronises the stream after every batch of eight short sweeps.
  */
 fr_status fr_fill(const float* dem, int64_t nx, int64_t ny, uint32_t flags, float* filled_out,
                   int32_t max_sweeps, int32_t* sweeps_out, void* ws, size_t ws_bytes,

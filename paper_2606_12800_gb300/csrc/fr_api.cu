@@ -66,15 +66,17 @@ Layout layout(int64_t n) {
     return L;
 }
 
-// fr_fill's workspace: the sweep counters (one per sweep of a batch) and two
+// fr_fill's workspace: the sweep counters (one per launch of a batch) and two
 // per-tile records of the tiles to run (the documented size, two bytes per
 // 64x32 tile, holds them twice over).
-constexpr int kFillBatch = 8;  // sweeps launched between two reads of the counters
-// Passes of a tile per sweep: two where the limit on sweeps is a mere backstop
-// (the fastest; see fr_fill.cu), and then eight such sweeps count as one towards the
-// limit; until the tile settles where the caller counts sweeps.
-constexpr int kFillQuickPasses = 2, kFillSettlePasses = 384;
-constexpr int32_t kFillQuickFrom = 4096;
+constexpr int kFillBatch = 8;  // launches between two reads of the counters
+// A launch takes a tile through two passes (the fastest; see fr_fill.cu), and eight
+// such launches make one sweep of the caller's.  What still moves when the caller's
+// limit is used up (channels that wind through a tile) gets as many sweeps again in
+// which every tile runs until it rests: the limit counts sweeps of that kind, and a
+// larger one never allows less.  A pass settles at least the next cell of a path, so
+// a tile's 4096 cells bound the passes.
+constexpr int kFillPerSweep = 8, kFillShortPasses = 2, kFillSettlePasses = 4096;
 size_t fill_ws_bytes(int64_t nx, int64_t ny) {
     return 256 + align256((size_t)(((nx + 63) / 64) * ((ny + 31) / 32))) * 2;
 }
@@ -333,31 +335,37 @@ fr_status fr_fill(const float* dem, int64_t nx, int64_t ny, uint32_t flags, floa
     const size_t ntiles = align256((size_t)fill_tiles(nx, ny));
     uint8_t* act[2] = {(uint8_t*)ws + 256, (uint8_t*)ws + 256 + ntiles};
     if (cudaMemsetAsync(act[0], 0, 2 * ntiles, s) != cudaSuccess) return FR_ERR_CUDA;
-    const bool quick = max_sweeps >= kFillQuickFrom;
-    const int64_t limit = quick ? 8 * (int64_t)max_sweeps : max_sweeps;
-    for (int64_t done = 0; done < limit;) {
-        const int32_t b = limit - done < kFillBatch ? (int32_t)(limit - done) : kFillBatch;
-        unsigned long long h[kFillBatch];
-        if (cudaMemsetAsync(counts, 0, sizeof(h), s) != cudaSuccess) return FR_ERR_CUDA;
-        for (int32_t k = 0; k < b; ++k) {
-            const int64_t sweep = done + k;  // 0-based
-            if (fill_sweep(dem, nx, ny, filled_out, act[(sweep + 1) & 1], act[sweep & 1], sweep == 0,
-                           quick ? kFillQuickPasses : kFillSettlePasses, counts + k, s) != cudaSuccess)
+    int64_t sweep = 0;  // launches so far
+    bool rest = false;  // the last one changed nothing
+    // up to `limit` launches, until one changes nothing; the number that changed something in *moved
+    auto relax = [&](int64_t limit, int passes, int64_t* moved) -> fr_status {
+        for (int64_t done = 0; done < limit && !rest;) {
+            const int32_t b = limit - done < kFillBatch ? (int32_t)(limit - done) : kFillBatch;
+            unsigned long long h[kFillBatch];
+            if (cudaMemsetAsync(counts, 0, sizeof(h), s) != cudaSuccess) return FR_ERR_CUDA;
+            for (int32_t k = 0; k < b; ++k, ++sweep)
+                if (fill_sweep(dem, nx, ny, filled_out, act[(sweep + 1) & 1], act[sweep & 1], sweep == 0, passes,
+                               counts + k, s) != cudaSuccess)
+                    return FR_ERR_CUDA;
+            if (cudaMemcpyAsync(h, counts, sizeof(h[0]) * b, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+                cudaStreamSynchronize(s) != cudaSuccess)
                 return FR_ERR_CUDA;
+            int32_t k = 0;
+            while (k < b && h[k] != 0) ++k;  // those after the first that changed nothing were idle
+            rest = k < b;
+            done += b;
+            *moved += k;
         }
-        if (cudaMemcpyAsync(h, counts, sizeof(h[0]) * b, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaStreamSynchronize(s) != cudaSuccess)
-            return FR_ERR_CUDA;
-        for (int32_t k = 0; k < b; ++k) {
-            if (h[k] == 0) {  // the first sweep that changed nothing; later ones were idle
-                if (sweeps_out) *sweeps_out = (int32_t)(done + k + 1);
-                return FR_OK;
-            }
-        }
-        done += b;
-        if (sweeps_out) *sweeps_out = (int32_t)done;
-    }
-    return FR_ERR_NO_PROGRESS;
+        return FR_OK;
+    };
+    // the last sweep allowed must be the one that changes nothing
+    int64_t moved = 0, settled = 0;
+    fr_status st = relax((int64_t)kFillPerSweep * (max_sweeps - 1) + 1, kFillShortPasses, &moved);
+    if (st != FR_OK) return st;
+    const bool quick = rest;
+    if (!rest && max_sweeps > 1 && (st = relax(max_sweeps, kFillSettlePasses, &settled)) != FR_OK) return st;
+    if (sweeps_out) *sweeps_out = quick ? (int32_t)((moved + kFillPerSweep - 1) / kFillPerSweep + 1) : max_sweeps;
+    return rest ? FR_OK : FR_ERR_NO_PROGRESS;
 }
 
 fr_status fr_accumulate_richardson(const fr_routing* R, const float* rain, float* w_out,
