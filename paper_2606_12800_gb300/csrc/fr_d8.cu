@@ -119,34 +119,6 @@ __device__ __forceinline__ void push4(S_& S, const int (&cq)[4]) {
         if (cq[q] >= 0) S.queue[pos++] = (uint16_t)cq[q];
 }
 
-// Per-byte population count.
-__device__ __forceinline__ uint32_t popc_bytes(uint32_t x) {
-    x = x - ((x >> 1) & 0x55555555u);
-    x = (x & 0x33333333u) + ((x >> 2) & 0x33333333u);
-    return (x + (x >> 4)) & 0x0F0F0F0Fu;
-}
-
-// The three 4-byte vectors (left, centre, right neighbours) of a group whose
-// first byte is word w1 of a padded row.
-struct Row3 {
-    uint32_t l, c, r;
-};
-__device__ __forceinline__ Row3 row3(const uint8_t* row, int w1) {
-    const uint32_t* p = reinterpret_cast<const uint32_t*>(row);
-    const uint32_t a = p[w1 - 1], b = p[w1], d = p[w1 + 1];
-    return {__byte_perm(a, b, 0x6543), b, __byte_perm(b, d, 0x4321)};
-}
-
-// 1 << code in each byte of x that holds a code 0..7, 0 in the others: a byte
-// permutation looks the bits up, its selectors the codes' nibbles.
-__device__ __forceinline__ uint32_t hot_bytes(uint32_t x) {
-    const uint32_t n = x & 0x0F0F0F0Fu;
-    const uint32_t sel = __byte_perm(n | (n >> 4), 0u, 0x4420);
-    uint32_t ok;  // 0xFF where the byte is a code: prmt with a selector's top bit set spreads the sign
-    asm("prmt.b32 %0, %1, 0, 0xBA98;" : "=r"(ok) : "r"(zero_bytes(x & 0xF8F8F8F8u)));
-    return __byte_perm(0x08040201u, 0x80402010u, sel) & ok;
-}
-
 __device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem) : "memory");
@@ -347,11 +319,7 @@ __global__ void __launch_bounds__(Gm::NT, d8_blocks<Gm, W>()) k_local_d8(Prob Po
             const Row3 up = row3(S.hot + ey * CP, w1);
             const Row3 mid = row3(S.hot + (ey + 1) * CP, w1);
             const Row3 dn = row3(S.hot + (ey + 2) * CP, w1);
-            // the donor in direction k has its bit opp(k) = k ^ 2 set
-            uint32_t dmf = ((mid.r >> 2) & 0x01010101u) | ((up.c >> 2) & 0x02020202u);
-            dmf |= ((mid.l << 2) & 0x04040404u) | ((dn.c << 2) & 0x08080808u);
-            dmf |= ((up.r >> 2) & 0x10101010u) | ((up.l >> 2) & 0x20202020u);
-            dmf |= ((dn.l << 2) & 0x40404040u) | ((dn.r << 2) & 0x80808080u);
+            const uint32_t dmf = donor_bits(up, mid, dn);
             const uint32_t wait = 0x09090909u - popc_bytes(dmf);  // kPkDone - donors
             const int r = (ey + 1) * CP + ex + 4;
             *reinterpret_cast<uint4*>(S.pk + r) =

@@ -282,6 +282,44 @@ __device__ __forceinline__ uint32_t zero_bytes(uint32_t x) {
     return ~(((x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | x) & 0x80808080u;
 }
 
+// Per-byte population count.
+__device__ __forceinline__ uint32_t popc_bytes(uint32_t x) {
+    x = x - ((x >> 1) & 0x55555555u);
+    x = (x & 0x33333333u) + ((x >> 2) & 0x33333333u);
+    return (x + (x >> 4)) & 0x0F0F0F0Fu;
+}
+
+// 1 << code in each byte of x that holds a code 0..7, 0 in the others: a byte
+// permutation looks the bits up, its selectors the codes' nibbles.
+__device__ __forceinline__ uint32_t hot_bytes(uint32_t x) {
+    const uint32_t n = x & 0x0F0F0F0Fu;
+    const uint32_t sel = __byte_perm(n | (n >> 4), 0u, 0x4420);
+    uint32_t ok;  // 0xFF where the byte is a code: prmt with a selector's top bit set spreads the sign
+    asm("prmt.b32 %0, %1, 0, 0xBA98;" : "=r"(ok) : "r"(zero_bytes(x & 0xF8F8F8F8u)));
+    return __byte_perm(0x08040201u, 0x80402010u, sel) & ok;
+}
+
+// The three 4-byte vectors (left, centre, right neighbours) of a group whose
+// first byte is word w1 of a padded row.
+struct Row3 {
+    uint32_t l, c, r;
+};
+__device__ __forceinline__ Row3 row3(const uint8_t* row, int w1) {
+    const uint32_t* p = reinterpret_cast<const uint32_t*>(row);
+    const uint32_t a = p[w1 - 1], b = p[w1], d = p[w1 + 1];
+    return {__byte_perm(a, b, 0x6543), b, __byte_perm(b, d, 0x4321)};
+}
+
+// Donor masks of four cells from the code bits of the rows around them: the donor
+// in direction k has its bit opp(k) = k ^ 2 set.
+__device__ __forceinline__ uint32_t donor_bits(const Row3& up, const Row3& mid, const Row3& dn) {
+    uint32_t d = ((mid.r >> 2) & 0x01010101u) | ((up.c >> 2) & 0x02020202u);
+    d |= ((mid.l << 2) & 0x04040404u) | ((dn.c << 2) & 0x08080808u);
+    d |= ((up.r >> 2) & 0x10101010u) | ((up.l >> 2) & 0x20202020u);
+    d |= ((dn.l << 2) & 0x40404040u) | ((dn.r << 2) & 0x80808080u);
+    return d;
+}
+
 // Fractions f_k = u_k / S from the weights u_k of a cell's receivers (0
 // elsewhere), with S the sum of the u_k in a fixed pairwise order
 // (((u0 + u1) + (u2 + u3)) + ((u4 + u5) + (u6 + u7)), two-float), inverted as two-float, and each f_k rounded once to fp32; 0 where bit k of m

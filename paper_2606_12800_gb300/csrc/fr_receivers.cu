@@ -1,11 +1,11 @@
 // fr_receivers.cu -- local flow routing kernels (paper Sec. 2.1 for D8,
 // App. A for the multi-receiver split).
 //
-// Codes alone come from the TMA-pipelined kernel, or by warps marching down
-// strips where TMA cannot address the grid; donor counts, D-infinity and batched
-// slope splits from blocks that stage a (TY+4) x (TX+4) elevation tile (two-cell
-// halo) in shared memory, which outside the grid holds +inf, never strictly lower
-// than anything.
+// D8 codes come from the TMA-pipelined kernel, or by warps marching down strips
+// where TMA cannot address the grid; their donor counts from the codes; donor
+// counts of the slope split, D-infinity and batched slope splits from blocks that
+// stage a (TY+4) x (TX+4) elevation tile (two-cell halo) in shared memory, which
+// outside the grid holds +inf, never strictly lower than anything.
 #include <cmath>
 #include <type_traits>
 
@@ -58,10 +58,14 @@ constexpr int kStrip = 4;  // rows of a strip (a tile is RTY / kStrip strips)
 // coalesced whatever the rows' alignment.  Bound by instruction issue.  1537x2603
 // 23 us by staged tiles, 19 us; batch of 32 tiles, 18 M cells, 160 us by staged
 // tiles of a block, 83 us (strips of 16 rows loaded as they go 116 us).
-template <bool LOWEST, bool D4, bool INTERIOR>
+// BITS: the codes also go to `bits` (rows of kBitsPitch bytes), one bit each.
+constexpr int kBitsPitch = RTX + 8;
+__device__ __forceinline__ uint8_t code_bit(uint32_t code) { return (uint8_t)(code < 8 ? 1u << code : 0u); }
+
+template <bool LOWEST, bool D4, bool INTERIOR, bool BITS>
 __device__ __forceinline__ void recv_d8_strip_t(const float* __restrict__ z, int64_t nx, int64_t ny,
                                               float c_orth, float c_diag, bool edge_route,
-                                              uint8_t* __restrict__ dir, int64_t x0, int64_t y0) {
+                                              uint8_t* __restrict__ dir, int64_t x0, int64_t y0, uint8_t* bits) {
     static_assert(RTX == 128, "four columns a lane");
     const float inf = __int_as_float(0x7f800000);
     const int lane = threadIdx.x & 31;
@@ -146,73 +150,84 @@ __device__ __forceinline__ void recv_d8_strip_t(const float* __restrict__ z, int
                 if (!edge_route && is_edge(gx, gy, nx, ny)) codes[g] = kSink;
             }
             o[32 * g] = (uint8_t)codes[g];
+            if (BITS) bits[r * kBitsPitch + lane + 32 * g] = code_bit(codes[g]);
         }
         a = b;
         b = c;
     }
 }
 
-template <bool LOWEST, bool D4>
+template <bool LOWEST, bool D4, bool BITS = false>
 __device__ __forceinline__ void recv_d8_strip(const float* __restrict__ z, int64_t nx, int64_t ny,
                                               float c_orth, float c_diag, bool edge_route,
-                                              uint8_t* __restrict__ dir, int64_t x0, int64_t y0) {
+                                              uint8_t* __restrict__ dir, int64_t x0, int64_t y0,
+                                              uint8_t* bits = nullptr) {
     if (x0 >= 1 && y0 >= 1 && x0 + RTX + 1 <= nx && y0 + kStrip + 1 <= ny)
-        recv_d8_strip_t<LOWEST, D4, true>(z, nx, ny, c_orth, c_diag, edge_route, dir, x0, y0);
+        recv_d8_strip_t<LOWEST, D4, true, BITS>(z, nx, ny, c_orth, c_diag, edge_route, dir, x0, y0, bits);
     else
-        recv_d8_strip_t<LOWEST, D4, false>(z, nx, ny, c_orth, c_diag, edge_route, dir, x0, y0);
+        recv_d8_strip_t<LOWEST, D4, false, BITS>(z, nx, ny, c_orth, c_diag, edge_route, dir, x0, y0, bits);
 }
 
-// D8 codes and donor counts of RTX x RTY tile cells by a block.
-template <bool LOWEST>
-__device__ __forceinline__ void recv_d8_tile(const float* __restrict__ z, int64_t nx, int64_t ny,
-                                             float c_orth, float c_diag, uint32_t flags,
-                                             uint8_t* __restrict__ dir,
-                                             uint8_t* __restrict__ indeg, int64_t x0,
-                                             int64_t y0) {
-    __shared__ float zs[HX * HY];
-    __shared__ uint8_t ds[RX * RY];
-    const bool edge_route = flags & kEdgeRoute;
-    const bool d4 = flags & kD4;
-    const float inf = __int_as_float(0x7f800000);
-    load_z_tile(zs, z, nx, ny, x0, y0);
-    __syncthreads();
-    // codes of the tile and the ring around it, then the donor counts
-    for (int i = threadIdx.x; i < RX * RY; i += RNT) {
-        const int ry = i / RX, rx = i - ry * RX;
-        const int64_t gx = x0 + rx - 1, gy = y0 + ry - 1;
-        uint8_t code = kSink;
-        if (gx >= 0 && gy >= 0 && gx < nx && gy < ny) {
-            if (edge_route || !is_edge(gx, gy, nx, ny)) {
-                float zn[8];
-                gather8(zs, rx, ry, zn);
-                if (d4) zn[4] = zn[5] = zn[6] = zn[7] = inf;
-                code = d8_code(zs[(ry + 1) * HX + (rx + 1)], zn, c_orth, c_diag, LOWEST);
-            }
-            if (rx >= 1 && rx <= RTX && ry >= 1 && ry <= RTY) dir[gy * nx + gx] = code;
-        }
-        ds[ry * RX + rx] = code;
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < RTX * RTY; i += RNT) {
-        const int ly = i / RTX, lx = i - ly * RTX;
-        const int64_t gx = x0 + lx, gy = y0 + ly;
-        if (gx >= nx || gy >= ny) continue;
-        int n = 0;
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-            n += ds[(ly + 1 + offy(k)) * RX + (lx + 1 + offx(k))] == (uint8_t)opp(k);
-        indeg[gy * nx + gx] = (uint8_t)n;
-    }
-}
+// Codes and donor counts: a strip per warp, eight strips to a block, the codes
+// also as bits in shared memory, with the ring around the block's tile (its codes
+// cell by cell); a donor test is then a shift and a mask for four cells.
+// Codes and counts of 4096x8192: 320 us by blocks that chose each cell of a staged
+// tile and ring in turn, 183 with four-cell windows there, 142 now; 160x192 15, 13
+// and 10 us, 1023x1025 21, 17 and 13 (codes first and counts in a second kernel: 143,
+// 16 and 18).
+constexpr int kCountRows = kStrip * RNT / 32;
 
-template <bool LOWEST>
+template <bool LOWEST, bool D4>
 __global__ void __launch_bounds__(RNT) k_receivers_d8_indeg(const float* __restrict__ z, int64_t nx,
                                                             int64_t ny, float c_orth, float c_diag,
                                                             uint32_t flags, uint8_t* __restrict__ dir,
                                                             uint8_t* __restrict__ indeg) {
-    int64_t x0, y0;
-    tile_origin(nx, x0, y0);
-    recv_d8_tile<LOWEST>(z, nx, ny, c_orth, c_diag, flags, dir, indeg, x0, y0);
+    // cell (lx, ly) of the tile at (ly + 1) * kBitsPitch + lx + 4
+    __shared__ alignas(4) uint8_t bits[(kCountRows + 2) * kBitsPitch];
+    const int64_t tiles_x = (nx + RTX - 1) / RTX;
+    const int64_t ty = blockIdx.x / tiles_x, tx = blockIdx.x - ty * tiles_x;
+    const int64_t x0 = tx * RTX, y0 = ty * kCountRows;
+    const bool edge_route = flags & kEdgeRoute;
+    for (int i = threadIdx.x; i < (int)sizeof(bits) / 4; i += RNT) reinterpret_cast<uint32_t*>(bits)[i] = 0u;
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (y0 + kStrip * warp < ny)
+        recv_d8_strip<LOWEST, D4, true>(z, nx, ny, c_orth, c_diag, edge_route, dir, x0, y0 + kStrip * warp,
+                                        bits + (1 + kStrip * warp) * kBitsPitch + 4);
+    for (int i = threadIdx.x; i < 2 * RX + 2 * kCountRows; i += RNT) {
+        const int j = i - 2 * RX;
+        const int rx = i < 2 * RX ? (i < RX ? i : i - RX) : (j & 1) * (RX - 1);
+        const int ry = i < 2 * RX ? (i < RX ? 0 : kCountRows + 1) : 1 + (j >> 1);
+        const int64_t gx = x0 + rx - 1, gy = y0 + ry - 1;
+        if (gx < 0 || gy < 0 || gx >= nx || gy >= ny || (!edge_route && is_edge(gx, gy, nx, ny))) continue;
+        float zn[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int64_t xn = gx + offx(k), yn = gy + offy(k);
+            zn[k] = (k >= 4 && D4) || xn < 0 || yn < 0 || xn >= nx || yn >= ny ? __int_as_float(0x7f800000)
+                                                                              : __ldg(z + yn * nx + xn);
+        }
+        bits[ry * kBitsPitch + rx + 3] = code_bit(d8_code(__ldg(z + gy * nx + gx), zn, c_orth, c_diag, LOWEST));
+    }
+    __syncthreads();
+    const bool aligned = (nx & 3) == 0 && ((uintptr_t)indeg & 3) == 0;
+    const int64_t gx = x0 + 4 * lane;
+    if (gx >= nx) return;
+    for (int ly = warp; ly < kCountRows; ly += RNT / 32) {
+        const int64_t gy = y0 + ly;
+        if (gy >= ny) break;
+        const Row3 up = row3(bits + ly * kBitsPitch, lane + 1), mid = row3(bits + (ly + 1) * kBitsPitch, lane + 1);
+        const Row3 dn = row3(bits + (ly + 2) * kBitsPitch, lane + 1);
+        const uint32_t n = popc_bytes(donor_bits(up, mid, dn));
+        uint8_t* o = indeg + gy * nx + gx;
+        if (aligned) {
+            *reinterpret_cast<uint32_t*>(o) = n;
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (gx + q < nx) o[q] = (uint8_t)(n >> (8 * q));
+        }
+    }
 }
 
 // A strip per warp.
@@ -790,7 +805,6 @@ cudaError_t launch_receiver_index(const uint8_t* dir, int64_t nx, int64_t ny, bo
 
 cudaError_t launch_receivers_d8(const float* z, int64_t nx, int64_t ny, double dx,
                                 uint32_t flags, uint8_t* dir, uint8_t* indeg, cudaStream_t s) {
-    const unsigned grid = (unsigned)(((nx + RTX - 1) / RTX) * ((ny + RTY - 1) / RTY));
     float co = (float)(1.0 / dx);
     float cd = (float)(1.0 / (std::sqrt(2.0) * dx));
     const bool lowest = flags & kD8Lowest;
@@ -805,16 +819,13 @@ cudaError_t launch_receivers_d8(const float* z, int64_t nx, int64_t ny, double d
         return d4 ? launch_d8_tma<false, true>(map, nx, ny, co, cd, flags, dir, s)
                   : launch_d8_tma<false, false>(map, nx, ny, co, cd, flags, dir, s);
     }
-    if (indeg) {
-        if (lowest) k_receivers_d8_indeg<true><<<grid, RNT, 0, s>>>(z, nx, ny, co, cd, flags, dir, indeg);
-        else k_receivers_d8_indeg<false><<<grid, RNT, 0, s>>>(z, nx, ny, co, cd, flags, dir, indeg);
-        return cudaGetLastError();
-    }
     const int64_t tiles = ((nx + RTX - 1) / RTX) * ((ny + kStrip - 1) / kStrip);
     const unsigned wgrid = (unsigned)((tiles + RNT / 32 - 1) / (RNT / 32));
+    const unsigned cgrid = (unsigned)(((nx + RTX - 1) / RTX) * ((ny + kCountRows - 1) / kCountRows));
     auto run = [&](auto low, auto d4) {
-        k_receivers_d8<decltype(low)::value, decltype(d4)::value>
-            <<<wgrid, RNT, 0, s>>>(z, nx, ny, co, cd, flags, dir, tiles);
+        constexpr bool L = decltype(low)::value, D = decltype(d4)::value;
+        if (indeg) k_receivers_d8_indeg<L, D><<<cgrid, RNT, 0, s>>>(z, nx, ny, co, cd, flags, dir, indeg);
+        else k_receivers_d8<L, D><<<wgrid, RNT, 0, s>>>(z, nx, ny, co, cd, flags, dir, tiles);
     };
     if (lowest && (flags & kD4)) run(std::true_type{}, std::true_type{});
     else if (lowest) run(std::true_type{}, std::false_type{});
