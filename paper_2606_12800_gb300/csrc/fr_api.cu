@@ -145,9 +145,9 @@ Prob base_prob(const fr_routing* R, char* ws, bool with_water = false, bool with
     P.glist = reinterpret_cast<unsigned long long*>(ws + L.glist);
     P.glist_cap = R->nx * R->ny;
     P.out_lo = reinterpret_cast<float*>(ws + L.lo);
-    // the skeleton solve's scratch shares the global-cell list's region (the
-    // list itself is read only by the cell walkers): walker starts, dependency
-    // slots
+    // the skeleton solve's scratch shares the global-cell list's region (polling
+    // and the cell walkers, which read the list, leave those cells to it): walker
+    // starts, dependency slots
     P.skel_min = ~0ull;
     if (R->kind == FR_ROUTING_D8) {
         const int side = skel_side(with_water, with_area, R->nx, R->ny);

@@ -606,6 +606,12 @@ __global__ void __launch_bounds__(256) k_global_levels(const Prob* __restrict__ 
 // arrival) took 41 us on 160x192, 56 on 1537x2603 and 57 on 4096^2, polling 17,
 // 25 and 23 us.
 //
+// Four cells a lane is also where the list ends on filled terrain and planes, whose
+// chains are as long as the grid: filled 1024^2 to 2048^2 (up to 210 K cells), forced
+// cell by cell, 4.9 to 12.5 ms with the walkers, 1.9 to 5.3 by polling; a plane of
+// 400x700 (280 K) 3.3 and 1.9, of 128x4000 (512 K) 18.5 and 12.4; slope split on filled
+// 2048^2 27.3 ms in rounds, 7.8 by polling, its adjoint on the 400x700 plane 7.2 and 2.3.
+//
 // A lane tries its cells in turn and never waits at one, and the launch is
 // cooperative (every lane runs), so an acyclic routing always gets on.  Where
 // nothing has been finished anywhere for kPollStuck tries (a cycle), or (MFD and
@@ -778,7 +784,7 @@ __global__ void __launch_bounds__(256) k_global_poll(const Prob* __restrict__ pr
         done += got;
         const unsigned n = __reduce_add_sync(0xffffffffu, got);
         if (n) {
-            if ((threadIdx.x & 31) == 0) atomicAdd(&G->rounds, (unsigned long long)n);  // cells finished so far
+            if ((threadIdx.x & 31) == 0) atomicAdd(&G->polled, (unsigned long long)n);  // cells finished so far
             stuck = 0;
             continue;
         }
@@ -786,7 +792,7 @@ __global__ void __launch_bounds__(256) k_global_poll(const Prob* __restrict__ pr
         int stop = 0;
         if ((threadIdx.x & 31) == 0) {
             if ((stuck & 63u) == 0) {
-                const unsigned long long now = global_ns(), all = ld_relaxed_u64(&G->rounds);
+                const unsigned long long now = global_ns(), all = ld_relaxed_u64(&G->polled);
                 if (all != seen) {
                     seen = all;
                     since = now;

@@ -63,8 +63,8 @@ struct EngineGlobals {
     unsigned long long fcount[3];    // level-synchronous global phase: frontier sizes
     unsigned int bar_count;          // grid barrier: blocks arrived
     unsigned int bar_gen;            // grid barrier: generation
-    unsigned long long rounds;       // polling: cells finished so far; level-synchronous phase: rounds run
-    unsigned long long unused;       // keeps the words behind it in place
+    unsigned long long rounds;       // level-synchronous global phase: rounds run
+    unsigned long long polled;       // polling: cells finished so far
     unsigned long long sink_area;    // D8 areas: sum of the areas of the FR_SINK cells the local phase finished
     unsigned long long pad[2];
 };
@@ -76,9 +76,10 @@ enum class Mode : int { FwdD8 = 0, FwdMfd = 1, AdjD8 = 2, AdjMfd = 3 };
 int walker_grid();
 // Blocks of the walker kernels on n cells: half the grid up to 2^24 cells, where
 // an idle launch is the usual case and the walkers gain nothing from more (filled
-// 4096^2 19.1 ms either way); all of it above 2^25, where a thread that follows a
-// trunk keeps its other starts waiting (filled 32768^2, forced walkers, half the
-// grid 1043 ms, all of it 370 to 615 from call to call).
+// terrain and planes, forced, 1500^2 to 5793^2: within 1 % of one another with all of
+// it, half and a quarter); all of it above 2^25, where a thread that follows a trunk
+// keeps its other starts waiting (filled 8192^2 61, 96 and 108 ms, 12000^2 102, 156
+// and 240; planes 57, 57 and 58, 73, 73 and 74).
 inline unsigned walker_blocks(unsigned long long n) {
     const unsigned all = (unsigned)walker_grid(), half = all / 2;
     const unsigned long long want = n >> 15;

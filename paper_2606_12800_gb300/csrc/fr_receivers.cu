@@ -35,13 +35,6 @@ __device__ __forceinline__ void load_z_tile(float* zs, const float* __restrict__
     }
 }
 
-// Neighbour elevations of ring-tile cell (rx, ry) (ring coordinates: tile
-// cell (0,0) is (1,1)).
-__device__ __forceinline__ void gather8(const float* zs, int rx, int ry, float (&zn)[8]) {
-#pragma unroll
-    for (int k = 0; k < 8; ++k) zn[k] = zs[(ry + 1 + offy(k)) * HX + (rx + 1 + offx(k))];
-}
-
 __device__ __forceinline__ void tile_origin(int64_t nx, int64_t& x0, int64_t& y0) {
     const int64_t tiles_x = (nx + RTX - 1) / RTX;
     const int64_t ty = blockIdx.x / tiles_x, tx = blockIdx.x - ty * tiles_x;
@@ -605,12 +598,12 @@ __global__ void __launch_bounds__(RNT) k_mfd_masks(const float* __restrict__ z, 
     }
 }
 
-// Fractions of given receiver masks (bits pointing off the grid are
-// ignored): one cell per thread, elevations staged like the receiver tiles.
-__global__ void __launch_bounds__(RNT) k_mfd_fractions(const float* __restrict__ z,
-                                                       const uint8_t* __restrict__ mask,
-                                                       int64_t nx, int64_t ny, MfdConst mc,
-                                                       uint32_t flags, float* __restrict__ frac) {
+// D-infinity fractions of given receiver masks (a cell with an empty mask gives
+// nothing): one cell per thread, elevations staged like the receiver tiles.
+__global__ void __launch_bounds__(RNT) k_dinf_fractions(const float* __restrict__ z,
+                                                        const uint8_t* __restrict__ mask,
+                                                        int64_t nx, int64_t ny, MfdConst mc,
+                                                        float* __restrict__ frac) {
     __shared__ float zs[HX * HY];
     int64_t x0, y0;
     tile_origin(nx, x0, y0);
@@ -622,20 +615,14 @@ __global__ void __launch_bounds__(RNT) k_mfd_fractions(const float* __restrict__
         if (gx >= nx || gy >= ny) continue;
         const int64_t gi = gy * nx + gx;
         if (!FR_OK(gi, nx * ny, 43)) continue;
-        const uint32_t m = mask[gi] & grid_mask8(gx, gy, nx, ny);
+        const uint32_t gm = grid_mask8(gx, gy, nx, ny);
         float zn[8], f[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) zn[k] = zs[(ly + 2 + offy(k)) * HX + (lx + 2 + offx(k))];
-        if (flags & kDinf) {
-            // the D-infinity split of this cell (its receivers are the mask's)
-            if (m) dinf_cell(zs[(ly + 2) * HX + (lx + 2)], zn, grid_mask8(gx, gy, nx, ny), mc.co_hi,
-                             mc.cd_hi, f);
-            else
-#pragma unroll
-                for (int k = 0; k < 8; ++k) f[k] = 0.0f;
-        } else {
-            mfd_fracs8(zs[(ly + 2) * HX + (lx + 2)], zn, m, mc, f);
+        for (int k = 0; k < 8; ++k) {
+            zn[k] = zs[(ly + 2 + offy(k)) * HX + (lx + 2 + offx(k))];
+            f[k] = 0.0f;
         }
+        if (mask[gi] & gm) dinf_cell(zs[(ly + 2) * HX + (lx + 2)], zn, gm, mc.co_hi, mc.cd_hi, f);
         float4* fo = reinterpret_cast<float4*>(frac + gi * 8);
         fo[0] = make_float4(f[0], f[1], f[2], f[3]);
         fo[1] = make_float4(f[4], f[5], f[6], f[7]);
@@ -874,7 +861,7 @@ cudaError_t launch_mfd_fractions(const float* z, const uint8_t* mask, int64_t nx
         return cudaGetLastError();
     }
     const unsigned grid = (unsigned)(((nx + RTX - 1) / RTX) * ((ny + RTY - 1) / RTY));
-    k_mfd_fractions<<<grid, RNT, 0, s>>>(z, mask, nx, ny, make_mfd_const(dx, p), flags, frac);
+    k_dinf_fractions<<<grid, RNT, 0, s>>>(z, mask, nx, ny, make_mfd_const(dx, p), frac);
     return cudaGetLastError();
 }
 
