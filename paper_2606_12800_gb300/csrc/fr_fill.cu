@@ -14,7 +14,8 @@
 // changes nothing: then every cell meets its equation, and the surface is the
 // unique solution, bit for bit.
 //
-// A sweep is one launch over 64x64 tiles.  A tile that has work loads F and z
+// A sweep here is one launch over 64x64 tiles (up to eight of them are one sweep
+// of the caller's).  A tile that has work loads F and z
 // with a one-cell ring into shared memory as integers ordered like the floats
 // (succ is then +1) and relaxes them in directional passes: warps run down,
 // up, right and left at once (two per direction, half the lines each), each

@@ -49,8 +49,8 @@ constexpr int kStrip = 4;  // rows of a strip (a tile is RTY / kStrip strips)
 // the rows with three rows in registers, neighbours along a row coming by
 // shuffles.  For grids TMA cannot address and for batches: every load is
 // coalesced whatever the rows' alignment.  Bound by instruction issue.  1537x2603
-// 23 us by staged tiles, 19 us; batch of 32 tiles, 18 M cells, 160 us by staged
-// tiles of a block, 83 us (strips of 16 rows loaded as they go 116 us).
+// 23 us by staged tiles, 16 us; batch of 32 tiles, 18 M cells, 160 us by staged
+// tiles of a block, 73 us (strips of 16 rows loaded as they go 116 us).
 // BITS: the codes also go to `bits` (rows of kBitsPitch bytes), one bit each.
 constexpr int kBitsPitch = RTX + 8;
 __device__ __forceinline__ uint8_t code_bit(uint32_t code) { return (uint8_t)(code < 8 ? 1u << code : 0u); }
@@ -243,8 +243,8 @@ __global__ void __launch_bounds__(RNT) k_receivers_d8(const float* __restrict__ 
 // multiple of 4, as TMA requires), so it is TTX + 8 wide.  The kernel is bound
 // by instruction issue and the ALU pipe (the eight directions' keys and their
 // selection): 32768^2 2.38 ms with a running best over the directions (66
-// instructions per cell), 2.04 ms with d8_code_max (56), 1.99 ms with two rows per
-// step (52).  128x64 tiles in
+// instructions per cell), 2.04 ms with d8_code_max (56), 1.92 ms with two rows per
+// step and zero keys settled by minima (51).  128x64 tiles in
 // two stages (three CTAs per SM) measured 4.7 % faster than 128x32 in three
 // (four CTAs per SM) at 32768^2: fewer halo rows and fewer per-tile waits and
 // barriers.
@@ -797,7 +797,8 @@ cudaError_t launch_receivers_d8(const float* z, int64_t nx, int64_t ny, double d
     const bool lowest = flags & kD8Lowest;
     // codes alone on a TMA-addressable grid that gives most SMs a tile: the
     // pipelined persistent kernel (below 2^20 cells the strips are the faster:
-    // 5 to 6 us against 7; 768^2 6.2 and 7.1, 1024^2 7.5 and 7.2, 2048^2 19 and 15)
+    // 512^2 5.8 us against 6.8, 768^2 6.5 and 7.0, 1024^2 7.0 and 7.2, 1280^2 11.0 and
+    // 9.2, 2048^2 18.9 and 14.4, 4096^2 54 and 37)
     CUtensorMap map;
     if (!indeg && nx * ny >= (int64_t)1 << 20 && encode_tile_map_f32(&map, z, nx, ny, TBX, TBY)) {
         const bool d4 = flags & kD4;
